@@ -166,6 +166,7 @@ int bfs_setup(const bfs_mesh *mesh, const bfs_topo *topo, double F, const bfs_op
     cudaGetDevice(&c->device);
     const int sms = bfs::num_sms(c->device);
     bfs::plans_for(c->Nt, c->Ns, o.src_splits, sms, &c->plan64, &c->plan32);
+    c->plan64 = bfs::plan64_fine(c->Nt, c->Ns, o.src_splits, sms);
     if (o.src_splits <= 0) {
         // FP32C: down to one chunk of sources per split while the split partial
         // sums stay below 2^20 target slots (40 MB): many short CTAs, so that the

@@ -30,12 +30,10 @@ constexpr int REC = 16;
 constexpr int TREC = 16;
 
 // Accumulators written by the pair kernels, per split and target:
-//   0  double layer at top targets (top and bottom sheets)
-//   1  single layer at top targets (top and bottom sheets)
-//   2  sum of w S2 at top targets
-//   3  double layer at bottom targets (top and bottom sheets)
-//   4  single layer of the top sheet at bottom targets
-constexpr int NACC = 5;
+//   0  double and single layers at top targets (top and bottom sheets)
+//   1  sum of w S2 at top targets
+//   2  double layers (both sheets) and single layer of the top sheet at bottom targets
+constexpr int NACC = 3;
 
 // One instance of a batched sweep as the persistent pair kernel sees it.
 struct BatchInst {
@@ -184,6 +182,8 @@ int residual_launch(bfs_ctx *c, const double *u, double *Fu, int precision, cuda
 int unpack_launch(bfs_ctx *c, const double *u, cudaStream_t s, int which = 3);
 int constB_launch(bfs_ctx *c, cudaStream_t s);
 PairPlan make_plan(int Nt, int Ns, int tpb, int tpt, int chunk, int splits_req, int sms);
+PairPlan fine_plan(int Nt, int Ns, int tpb, int unit, int per_sm, int splits_req, int sms);
+PairPlan plan64_fine(int Nt, int Ns, int splits_req, int sms);
 void plans_for(int Nt, int Ns, int splits_req, int sms, PairPlan *p64, PairPlan *p32);
 
 int finish_launch(bfs_ctx *c, double *Fu, int precision, cudaStream_t s);

@@ -259,7 +259,7 @@ k_pairs_df(const float *__restrict__ src, int per_split, const float *__restrict
         }
     }
     if (t >= Nt) return;
-    const df acc[NACC] = {aT1, aT2, aS, aB1, aB2};
+    const df acc[NACC] = {df_add(aT1, aT2), aS, df_add(aB1, aB2)};
 #pragma unroll
     for (int q = 0; q < NACC; q++)
         part[((size_t)split * NACC + q) * Nt + t] = (double)acc[q].hi + (double)acc[q].lo;

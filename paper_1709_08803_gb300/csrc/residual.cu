@@ -172,12 +172,21 @@ __global__ void k_records(double *nodal, const double *__restrict__ beta,
 // ---------------------------------------------------------------------------
 // All-pairs quadrature.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
-
-template <typename R> struct Vec;
-template <> struct Vec<float> { typedef float4 T; static constexpr int W = 4; };
-template <> struct Vec<double> { typedef double2 T; static constexpr int W = 2; };
+// 1/sqrt(a), FP64: the hardware seed (about 20 bits, one special-function
+// instruction) and one third-order step, y (1 + e/2 + 3 e^2/8) with
+// e = 1 - a y^2 (the binomial series of (1 - e)^(-1/2); what it drops is below
+// 2^-58).  Five FP64 instructions against the library call's eight, on a GPU
+// whose FP64 pipe retires two per clock and SM and bounds the FP64 pair sum.
+// a is at least 1/4 there (half-integer offsets in mesh units); an infinite a
+// gives 0 and a NaN gives NaN, as the library call does.
+__device__ __forceinline__ double rsq64(double a)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    double e = fma(-(a * y), y, 1.0);
+    if (__double2hiint(a) == 0x7ff00000) e = 0.0;
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
 
 // Knuth's two-sum: hi + lo == a + b exactly.
 __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float b)
@@ -189,120 +198,116 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float b)
     lo += err;
 }
 
-// One tile of the all-pairs sum: targets [tile * TPB * TPT, +TPB * TPT) against
-// the sources of split `split`; writes that split's partial sums.
-template <typename R, int TPB, int TPT, int CH, bool COMP>
-__device__ __forceinline__ void pair_tile(const R *__restrict__ src, int per_split,
-                                          const R *__restrict__ tgt, int Nt,
-                                          double *__restrict__ part, int tile, int split, R *sh)
+// One tile of the FP64 all-pairs sum: targets [tile * TPB * TPT, +TPB * TPT)
+// against the sources of split `split`; writes that split's partial sums.
+// Bound by the FP64 pipe, so what counts is FP64 instructions per index pair:
+// 70 (five reciprocal roots of 5 among them; 86 before).  The double and the
+// single layer of a pairing share one accumulation, ri (t ri^2 + w zeta_x), the
+// slope terms s zeta_x + t zeta_y are formed once per source sheet, and the S2
+// form is s^2 + t^2 + (zeta_x* s + zeta_y* t)^2 on the shared s^2 + t^2.
+// 181 x 61: 16.9 -> 14.8 ms per launch (the pipe's floor for 70 is 13.7 ms).
+template <int TPB, int TPT, int CH>
+__device__ __forceinline__ void pair_tile(const double *__restrict__ src, int per_split,
+                                          const double *__restrict__ tgt, int Nt,
+                                          double *__restrict__ part, int tile, int split, double *sh)
 {
-    typedef typename Vec<R>::T V;
-    constexpr int VW = Vec<R>::W;
-    const R *sb = src + (size_t)split * per_split * REC;
+    typedef double2 V;
+    constexpr int VW = 2;
+    const double *sb = src + (size_t)split * per_split * REC;
 
-    R tx[TPT], ty[TPT], tz[TPT], tB[TPT], tf[TPT], tg[TPT];
-    R cA[TPT], cB[TPT], cC[TPT], cTB[TPT], cBT[TPT];
+    double tx[TPT], ty[TPT], tz[TPT], tB[TPT], tf[TPT], tg[TPT];
+    double tzx[TPT], tzy[TPT], cTB[TPT], cBT[TPT];
     int tid[TPT];
 #pragma unroll
     for (int p = 0; p < TPT; p++) {
         int t = tile * TPB * TPT + p * TPB + threadIdx.x;
         tid[p] = t;
-        const R *tr = tgt + (size_t)min(t, Nt - 1) * TREC;
+        const double *tr = tgt + (size_t)min(t, Nt - 1) * TREC;
         tx[p] = tr[0]; ty[p] = tr[1]; tz[p] = tr[2]; tB[p] = tr[3];
-        tf[p] = tr[6]; tg[p] = tr[7]; cA[p] = tr[8]; cB[p] = tr[9]; cC[p] = tr[10];
+        tzx[p] = tr[4]; tzy[p] = tr[5]; tf[p] = tr[6]; tg[p] = tr[7];
         cTB[p] = tr[11]; cBT[p] = tr[12];
     }
-    R hi[TPT][NACC], lo[TPT][NACC];
+    double hi[TPT][NACC];
 #pragma unroll
     for (int p = 0; p < TPT; p++)
 #pragma unroll
-        for (int q = 0; q < NACC; q++) { hi[p][q] = R(0); lo[p][q] = R(0); }
+        for (int q = 0; q < NACC; q++) hi[p][q] = 0.0;
 
     for (int c0 = 0; c0 < per_split; c0 += CH) {
+        const int nc = min(CH, per_split - c0);
         __syncthreads();
         const V *g = reinterpret_cast<const V *>(sb + (size_t)c0 * REC);
         V *sv = reinterpret_cast<V *>(sh);
-        for (int e = threadIdx.x; e < CH * REC / VW; e += TPB) sv[e] = g[e];
+        for (int e = threadIdx.x; e < nc * REC / VW; e += TPB) sv[e] = g[e];
         __syncthreads();
-        R l[TPT][NACC];
+        double l[TPT][NACC];
 #pragma unroll
         for (int p = 0; p < TPT; p++)
 #pragma unroll
-            for (int q = 0; q < NACC; q++) l[p][q] = R(0);
+            for (int q = 0; q < NACC; q++) l[p][q] = 0.0;
 #pragma unroll 2
-        for (int s = 0; s < CH; s++) {
-            const R *r = sh + s * REC;
-            const R xs = r[0], ys = r[1], zs = r[2], bs = r[3];
-            const R zxs = r[4], zys = r[5], bxs = r[6], bys = r[7];
-            const R w1f = r[8], w2zx = r[9], w1g = r[10], w2sb = r[11];
-            const R w1 = r[12], w2 = r[13];
+        for (int s = 0; s < nc; s++) {
+            const double *r = sh + s * REC;
+            const double xs = r[0], ys = r[1], zs = r[2], bs = r[3];
+            const double zxs = r[4], zys = r[5], bxs = r[6], bys = r[7];
+            const double w1f = r[8], w2zx = r[9], w1g = r[10], w2sb = r[11];
+            const double w1 = r[12], w2 = r[13];
 #pragma unroll
             for (int p = 0; p < TPT; p++) {
-                const R sx = xs - tx[p], sy = ys - ty[p];
-                const R syy = sy * sy;
-                const R rho2 = fma(sx, sx, syy);
+                const double sx = xs - tx[p], sy = ys - ty[p];
+                const double rho2 = fma(sx, sx, sy * sy);
+                const double gt = fma(sy, zys, sx * zxs), gb = fma(sy, bys, sx * bxs);
                 // top target, top source: w (f - f*) K1 + w zeta_x K2, and w S2
                 {
-                    const R d = zs - tz[p];
-                    const R ri = rsq(fma(d, d, rho2));
-                    const R ri3 = ri * ri * ri;
-                    const R num = fma(-sy, zys, fma(-sx, zxs, d));
-                    const R dens = fma(-tf[p], w1, w1f);
-                    l[p][0] = fma(dens * num, ri3, l[p][0]);
-                    l[p][1] = fma(w2zx, ri, l[p][1]);
-                    const R qf = fma(sx, fma(cA[p], sx, cB[p] * sy), cC[p] * syy);
-                    l[p][2] = fma(w2, rsq(qf), l[p][2]);
+                    const double d = zs - tz[p];
+                    const double ri = rsq64(fma(d, d, rho2));
+                    const double t = fma(-tf[p], w1, w1f) * (d - gt);
+                    l[p][0] = fma(fma(t, ri * ri, w2zx), ri, l[p][0]);
+                    // A s^2 + B s t + C t^2 = s^2 + t^2 + (zeta_x* s + zeta_y* t)^2
+                    const double m = fma(tzy[p], sy, tzx[p] * sx);
+                    l[p][1] = fma(w2, rsq64(fma(m, m, rho2)), l[p][1]);
                 }
                 // top target, bottom source: -w g K1(beta) + w sigma beta_x K2(beta)
                 {
-                    const R d = bs - cTB[p];
-                    const R ri = rsq(fma(d, d, rho2));
-                    const R ri3 = ri * ri * ri;
-                    const R num = fma(-sy, bys, fma(-sx, bxs, d));
-                    l[p][0] = fma(-(w1g * num), ri3, l[p][0]);
-                    l[p][1] = fma(w2sb, ri, l[p][1]);
+                    const double d = bs - cTB[p];
+                    const double ri = rsq64(fma(d, d, rho2));
+                    const double t = w1g * (gb - d);
+                    l[p][0] = fma(fma(t, ri * ri, w2sb), ri, l[p][0]);
                 }
                 // bottom target, top source: w f K1 + w zeta_x K2
                 {
-                    const R d = zs - cBT[p];
-                    const R ri = rsq(fma(d, d, rho2));
-                    const R ri3 = ri * ri * ri;
-                    const R num = fma(-sy, zys, fma(-sx, zxs, d));
-                    l[p][3] = fma(w1f * num, ri3, l[p][3]);
-                    l[p][4] = fma(w2zx, ri, l[p][4]);
+                    const double d = zs - cBT[p];
+                    const double ri = rsq64(fma(d, d, rho2));
+                    const double t = w1f * (d - gt);
+                    l[p][2] = fma(fma(t, ri * ri, w2zx), ri, l[p][2]);
                 }
                 // bottom target, bottom source: -w (g - g*) K1(beta)
                 {
-                    const R d = bs - tB[p];
-                    const R ri = rsq(fma(d, d, rho2));
-                    const R ri3 = ri * ri * ri;
-                    const R num = fma(-sy, bys, fma(-sx, bxs, d));
-                    const R dens = fma(-tg[p], w1, w1g);
-                    l[p][3] = fma(-(dens * num), ri3, l[p][3]);
+                    const double d = bs - tB[p];
+                    const double ri = rsq64(fma(d, d, rho2));
+                    const double t = fma(-tg[p], w1, w1g) * (gb - d);
+                    l[p][2] = fma(t * (ri * ri), ri, l[p][2]);
                 }
             }
         }
 #pragma unroll
         for (int p = 0; p < TPT; p++)
 #pragma unroll
-            for (int q = 0; q < NACC; q++) {
-                if constexpr (COMP) two_sum_acc(hi[p][q], lo[p][q], l[p][q]);
-                else hi[p][q] += l[p][q];
-            }
+            for (int q = 0; q < NACC; q++) hi[p][q] += l[p][q];
     }
 #pragma unroll
     for (int p = 0; p < TPT; p++) {
         if (tid[p] >= Nt) continue;
 #pragma unroll
         for (int q = 0; q < NACC; q++)
-            part[((size_t)split * NACC + q) * Nt + tid[p]] = (double)hi[p][q] + (double)lo[p][q];
+            part[((size_t)split * NACC + q) * Nt + tid[p]] = hi[p][q];
     }
 }
 
 // ---------------------------------------------------------------------------
 // FP32C all-pairs with the packed FP32x2 arithmetic of sm_100-class GPUs: one
-// instruction applies the same operation to two sources, so the 45 FP32
-// operations of an index pair take 23 issue slots (the five reciprocal square
+// instruction applies the same operation to two sources, so the 42 FP32
+// operations of an index pair take 21 issue slots (the five reciprocal square
 // roots stay scalar on the special-function unit); the FMA pipe still spends
 // one lane-cycle per operation, and it is the kernel's limit.  The quadratic
 // form of S2 is taken as s^2 + t^2 + (zeta_x* s + zeta_y* t)^2 (three
@@ -477,41 +482,34 @@ __device__ __forceinline__ void pair_tile_x2(const float *__restrict__ src, int 
                 {
                     const f2 d = f2_sub(zs, TZ[p]);
                     const f2 ri = f2_rsq(f2_fma(d, d, rho2));
-                    const f2 ri3 = f2_mul(f2_mul(ri, ri), ri);
                     const f2 num = f2_fma(sy, zys, f2_fma(sx, zxs, d));
-                    const f2 dens = f2_fma(NTF[p], w1, w1f);
-                    L[p][0] = f2_fma(f2_mul(dens, num), ri3, L[p][0]);
-                    L[p][1] = f2_fma(w2zx, ri, L[p][1]);
+                    const f2 t = f2_mul(f2_fma(NTF[p], w1, w1f), num);
+                    L[p][0] = f2_fma(f2_fma(t, f2_mul(ri, ri), w2zx), ri, L[p][0]);
                     // A s^2 + B s t + C t^2 = s^2 + t^2 + (zeta_x* s + zeta_y* t)^2
                     const f2 mq = f2_fma(ZX[p], sx, f2_mul(ZY[p], sy));
-                    L[p][2] = f2_fma(w2, f2_rsq(f2_fma(mq, mq, rho2)), L[p][2]);
+                    L[p][1] = f2_fma(w2, f2_rsq(f2_fma(mq, mq, rho2)), L[p][1]);
                 }
                 // top target, bottom source: -w g K1(beta) + w sigma beta_x K2(beta)
                 {
                     const f2 d = f2_sub(bs, CTB[p]);
                     const f2 ri = f2_rsq(f2_fma(d, d, rho2));
-                    const f2 ri3 = f2_mul(f2_mul(ri, ri), ri);
                     const f2 num = f2_fma(sy, bys, f2_fma(sx, bxs, d));
-                    L[p][0] = f2_fma(f2_mul(nw1g, num), ri3, L[p][0]);
-                    L[p][1] = f2_fma(w2sb, ri, L[p][1]);
+                    L[p][0] = f2_fma(f2_fma(f2_mul(nw1g, num), f2_mul(ri, ri), w2sb), ri, L[p][0]);
                 }
                 // bottom target, top source: w f K1 + w zeta_x K2
                 {
                     const f2 d = f2_sub(zs, CBT[p]);
                     const f2 ri = f2_rsq(f2_fma(d, d, rho2));
-                    const f2 ri3 = f2_mul(f2_mul(ri, ri), ri);
                     const f2 num = f2_fma(sy, zys, f2_fma(sx, zxs, d));
-                    L[p][3] = f2_fma(f2_mul(w1f, num), ri3, L[p][3]);
-                    L[p][4] = f2_fma(w2zx, ri, L[p][4]);
+                    L[p][2] = f2_fma(f2_fma(f2_mul(w1f, num), f2_mul(ri, ri), w2zx), ri, L[p][2]);
                 }
                 // bottom target, bottom source: -w (g - g*) K1(beta)
                 {
                     const f2 d = f2_sub(bs, TB[p]);
                     const f2 ri = f2_rsq(f2_fma(d, d, rho2));
-                    const f2 ri3 = f2_mul(f2_mul(ri, ri), ri);
                     const f2 num = f2_fma(sy, bys, f2_fma(sx, bxs, d));
                     const f2 densn = f2_fma(TG[p], w1, nw1g);  // g* w - w g
-                    L[p][3] = f2_fma(f2_mul(densn, num), ri3, L[p][3]);
+                    L[p][2] = f2_fma(f2_mul(f2_mul(densn, num), f2_mul(ri, ri)), ri, L[p][2]);
                 }
             }
         }
@@ -537,21 +535,25 @@ __device__ __forceinline__ void pair_tile_x2(const float *__restrict__ src, int 
     }
 }
 
-template <typename R, int TPB, int TPT, int CH, bool COMP>
+template <int TPB, int TPT, int CH>
 __global__ void __launch_bounds__(TPB)
-k_pairs(const R *__restrict__ src, int per_split, const R *__restrict__ tgt, int Nt,
-        double *__restrict__ part, int *flag)
+k_pairs32(const float *__restrict__ src, int per_split, const float *__restrict__ tgt, int Nt,
+          double *__restrict__ part, int *flag)
 {
-    if constexpr (sizeof(R) == 4 && COMP) {
-        __shared__ __align__(128) float sh[2 * CH * REC];
-        __shared__ __align__(8) unsigned long long bar[2];
-        ChunkRing ring{sh, bar, 0u, (unsigned int)(CH * REC)};
-        chunk_ring_init(ring);
-        pair_tile_x2<TPB, TPT, CH>(src, per_split, tgt, Nt, part, blockIdx.x, blockIdx.y, ring, flag);
-    } else {
-        __shared__ __align__(16) R sh[CH * REC];
-        pair_tile<R, TPB, TPT, CH, COMP>(src, per_split, tgt, Nt, part, blockIdx.x, blockIdx.y, sh);
-    }
+    __shared__ __align__(128) float sh[2 * CH * REC];
+    __shared__ __align__(8) unsigned long long bar[2];
+    ChunkRing ring{sh, bar, 0u, (unsigned int)(CH * REC)};
+    chunk_ring_init(ring);
+    pair_tile_x2<TPB, TPT, CH>(src, per_split, tgt, Nt, part, blockIdx.x, blockIdx.y, ring, flag);
+}
+
+template <int TPB, int TPT, int CH>
+__global__ void __launch_bounds__(TPB, 5)
+k_pairs64(const double *__restrict__ src, int per_split, const double *__restrict__ tgt, int Nt,
+          double *__restrict__ part)
+{
+    __shared__ __align__(16) double sh[CH * REC];
+    pair_tile<TPB, TPT, CH>(src, per_split, tgt, Nt, part, blockIdx.x, blockIdx.y, sh);
 }
 
 // ---------------------------------------------------------------------------
@@ -719,8 +721,8 @@ __global__ void k_finish(const double *__restrict__ part, const double *__restri
     if (is_t && q4 == 0) {
         const double zs = r[2] * a.dx, zxs = r[4], zys = r[5], fs = r[6], gs = r[7];
         const double pxs = r[13], pys = r[14];
-        const double F2 = acc[0] + acc[1] - zxs * acc[2] + zxs * g2 - TWO_PI * fs;
-        const double F7 = acc[3] + acc[4] + constB[e] - TWO_PI * gs;
+        const double F2 = acc[0] - zxs * acc[1] + zxs * g2 - TWO_PI * fs;
+        const double F7 = acc[2] + constB[e] - TWO_PI * gs;
         const double num = (1.0 + zxs * zxs) * pys * pys + (1.0 + zys * zys) * pxs * pxs -
                            2.0 * zxs * zys * pxs * pys;
         double F1 = 0.5 * num / (1.0 + zxs * zxs + zys * zys) + zs * a.iF2 - 0.5;
@@ -845,6 +847,26 @@ PairPlan make_plan(int Nt, int Ns, int tpb, int tpt, int chunk, int splits_req, 
     return p;
 }
 
+// Source splits of the FP64 and double-float pair kernels (one target per
+// thread): about twelve CTAs for each of the GPU's resident ones, so that the
+// last wave is a small part of the launch, in units of `unit` sources, so that
+// a small mesh still spreads over the GPU; the partial sums stay within 2^20
+// target slots (25 MB, L2-resident).  splits_req > 0 asks for a split count.
+PairPlan fine_plan(int Nt, int Ns, int tpb, int unit, int per_sm, int splits_req, int sms)
+{
+    PairPlan p;
+    p.tpb = tpb; p.tpt = 1; p.chunk = unit;
+    p.tiles = (Nt + tpb - 1) / tpb;
+    const int units = (Ns + unit - 1) / unit;
+    int want = splits_req;
+    if (want <= 0) want = std::min((sms * per_sm * 12 + p.tiles - 1) / p.tiles, std::max(1, (1 << 20) / Nt));
+    want = std::min(std::max(want, 1), units);
+    const int ups = (units + want - 1) / want;
+    p.splits = (units + ups - 1) / ups;
+    p.per_split = ups * unit;
+    return p;
+}
+
 int unpack_launch(bfs_ctx *c, const double *u, cudaStream_t s, int which)
 {
     k_unpack<<<(3 * c->M * 32 + 127) / 128, 128, 0, s>>>(u, c->d_nodal, c->N, c->M, c->dx);
@@ -861,7 +883,7 @@ int unpack_launch(bfs_ctx *c, const double *u, cudaStream_t s, int which)
 }
 
 // Launch configurations of the pair kernels.
-constexpr int P64_TPB = 128, P64_TPT = 1, P64_CH = 32;
+constexpr int P64_TPB = 128, P64_TPT = 1, P64_CH = 32, P64_UNIT = 8;
 constexpr int P32_TPB = 128, P32_TPT = 2, P32_CH = 128;
 
 int residual_launch(bfs_ctx *c, const double *u, double *Fu, int precision, cudaStream_t s)
@@ -881,11 +903,11 @@ int residual_launch(bfs_ctx *c, const double *u, double *Fu, int precision, cuda
     if (precision == BFS_DF64) {
         if ((rc = pairs_df_launch(c, s))) return rc;
     } else if (precision == BFS_FP32C)
-        k_pairs<float, P32_TPB, P32_TPT, P32_CH, true>
+        k_pairs32<P32_TPB, P32_TPT, P32_CH>
             <<<grid, P32_TPB, 0, s>>>(c->d_src32, p.per_split, c->d_tgt32, c->Nt, c->d_part, c->d_flag);
     else
-        k_pairs<double, P64_TPB, P64_TPT, P64_CH, false>
-            <<<grid, P64_TPB, 0, s>>>(c->d_src64, p.per_split, c->d_tgt64, c->Nt, c->d_part, c->d_flag);
+        k_pairs64<P64_TPB, P64_TPT, P64_CH>
+            <<<grid, P64_TPB, 0, s>>>(c->d_src64, p.per_split, c->d_tgt64, c->Nt, c->d_part);
     if (precision != BFS_DF64) c->launches++;
     if (ev1) cudaEventRecord(ev1, s);
     FinArgs fa = fin_args(c, p.splits, precision == BFS_FP32C);
@@ -981,6 +1003,11 @@ cudaEvent_t prof_event(bfs_ctx *c)
         c->ev_pool.push_back(e);
     }
     return c->ev_pool[c->ev_used++];
+}
+
+PairPlan plan64_fine(int Nt, int Ns, int splits_req, int sms)
+{
+    return fine_plan(Nt, Ns, P64_TPB, P64_UNIT, 5, splits_req, sms);
 }
 
 void plans_for(int Nt, int Ns, int splits_req, int sms, PairPlan *p64, PairPlan *p32)
