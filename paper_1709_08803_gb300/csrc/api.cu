@@ -200,8 +200,8 @@ int bfs_setup(const bfs_mesh *mesh, const bfs_topo *topo, double F, const bfs_op
     ALLOC(c->d_src32, sizeof(float) * bfs::REC * (size_t)c->Ns_cap);
     ALLOC(c->d_tgt64, sizeof(double) * bfs::TREC * (size_t)c->Nt);
     ALLOC(c->d_tgt32, sizeof(float) * bfs::TREC * (size_t)c->Nt);
-    ALLOC(c->d_srcdf, sizeof(float) * 32 * (size_t)c->Ns_cap);
-    ALLOC(c->d_tgtdf, sizeof(float) * 32 * (size_t)c->Nt);
+    ALLOC(c->d_srcdf, sizeof(float) * bfs::DSRC * (size_t)c->Ns_cap);
+    ALLOC(c->d_tgtdf, sizeof(float) * bfs::DTGT * (size_t)c->Nt);
     ALLOC(c->d_part, sizeof(double) * c->part_cap);
     ALLOC(c->d_constB, sizeof(double) * (size_t)c->Nt);
     ALLOC(c->d_flag, sizeof(int));

@@ -29,6 +29,17 @@ constexpr int REC = 16;
 //   11 zeta*/dx + 1/dx   12 (beta*+1)/dx - 1/dx   13 phi_x*  14 phi_y*  15 unused
 constexpr int TREC = 16;
 
+// Double-float records of the df64 pair kernel (hi/lo float pairs from index 2
+// on; lengths in mesh units as above).  A source has DSRC floats, sources in
+// interleaved pairs:
+//   0 column  1 row (mesh units, exact)  2 zeta/dx  4 (beta+1)/dx
+//   6 zeta_x  8 zeta_y dy/dx  10 beta_x  12 beta_y dy/dx
+//   14 c f  16 c g  18 c dx zeta_x  20 c dx sigma beta_x  22 c  23 unused
+// with c = cx cy the trapezoid weight without dx dy.  A target has DTGT floats:
+//   0 column  1 row  2 zeta*/dx  4 zeta*/dx + 1/dx  6 (beta*+1)/dx - 1/dx
+//   8 (beta*+1)/dx  10 f*  12 g*  14 zeta_x*  16 zeta_y* dy/dx  18,19 unused
+constexpr int DSRC = 24, DTGT = 20;
+
 // Accumulators written by the pair kernels, per split and target:
 //   0  double and single layers at top targets (top and bottom sheets)
 //   1  sum of w S2 at top targets
@@ -102,8 +113,8 @@ struct bfs_ctx {
     double *d_constB;              // Nt: bottom-only single-layer part at bottom targets
     double *d_psurf;               // NM applied surface pressure, or nullptr
     int *d_flag;                   // non-finite flag
-    float *d_srcdf;                // Ns_cap * 32 double-float source records
-    float *d_tgtdf;                // Nt * 32 double-float target records
+    float *d_srcdf;                // Ns_cap * DSRC double-float source records
+    float *d_tgtdf;                // Nt * DTGT double-float target records
     bfs::PairPlan plan64, plan32, plandf;
     size_t part_cap;
 
@@ -179,6 +190,7 @@ namespace bfs {
 
 // residual.cu
 int residual_launch(bfs_ctx *c, const double *u, double *Fu, int precision, cudaStream_t s);
+// which: record copies to write, bit 0 FP64, bit 1 FP32, bit 2 double-float
 int unpack_launch(bfs_ctx *c, const double *u, cudaStream_t s, int which = 3);
 int constB_launch(bfs_ctx *c, cudaStream_t s);
 PairPlan make_plan(int Nt, int Ns, int tpb, int tpt, int chunk, int splits_req, int sms);
@@ -247,6 +259,55 @@ void precond_free(bfs_ctx *c);
 int num_sms(int device);
 // records an event pair around a pair-kernel launch when profiling is on
 cudaEvent_t prof_event(bfs_ctx *c);
+// Packed FP32x2 arithmetic of sm_100-class GPUs: one instruction applies the
+// same operation to two values (low and high half of a 64-bit register pair).
+struct f2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ f2 f2_pack(float a, float b)
+{
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void f2_unpack(f2 x, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c)
+{
+    f2 d;
+    asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(d.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return d;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b)
+{
+    f2 d;
+    asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
+    return d;
+}
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b)
+{
+    f2 d;
+    asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
+    return d;
+}
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b)
+{
+    f2 d;
+    asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
+    return d;
+}
+// sign flip of both halves: integer operations, off the FMA pipe
+__device__ __forceinline__ f2 f2_neg(f2 a) { return f2{a.v ^ 0x8000000080000000ull}; }
+__device__ __forceinline__ f2 f2_both(float a) { return f2_pack(a, a); }
+__device__ __forceinline__ f2 f2_rsq(f2 x)
+{
+    float a, b;
+    f2_unpack(x, a, b);
+    return f2_pack(rsqrtf(a), rsqrtf(b));
+}
+
 }  // namespace bfs
 
 #define BFS_CUDA_TRY(ctx, call)                                                      \

@@ -10,281 +10,258 @@
 // are the same four sheet pairings, singularity subtractions and S2 term as
 // the FP64 and FP32C kernels (Sec. 2.2 and 3.1 of the paper).
 //
-// Horizontal offsets are exact in single precision: records carry the node
-// column and row positions in mesh units (half-integers), the x offset is in
-// units of dx and the y offset is (row difference) * dy/dx, applied as a
-// double-float factor.
+// The kernel is bound by the FMA pipe (two sources per instruction, packed
+// FP32x2), so its cost is the number of FP32 operations per index pair: 321 on
+// meshes with dx == dy, about 370 otherwise (659 single instructions before).
+// 181 x 61: 2.29 -> 1.19 ms per launch with the pipe 82 % busy; 281 x 281:
+// 117 -> 60 ms.  Occupancies from 3 to 6 CTAs per SM measure the same within 1 %.
+// What keeps the count down:
+//   - Horizontal offsets are exact: records carry the node column and row in
+//     mesh units (half-integers), so with dx == dy s^2 + t^2 is one exact float
+//     (SQ), else an exact s^2 plus (dy/dx)^2 t^2 in double-float.
+//   - Weights cx cy (1, 1/2 or 1/4) are exact; the common factors dy/dx and dy
+//     are applied to the finished sums.
+//   - The slope terms s zeta_x + t zeta_y are formed once per source sheet.
+//   - 1/r, 1/r^2 share one residual e = 1 - a y0^2 of the FP32 seed y0:
+//     1/r = y0 (1 + e/2 + 3 e^2/8), 1/r^2 = y0^2 (1 + e + e^2).
+//   - Double and single layer of a pairing share one accumulation,
+//     (t / r^2 + w zeta_x) / r.
+// Renormalisation is left out inside a term: a low part may reach about 2^-22 of
+// the operands its high part came from.  The three accumulators, whose low parts
+// collect one rounding error per term, are renormalised every fourth source pair
+// (without that the 281 x 281 residual loses two bits).
 #include <math.h>
 
 #include "bfs_internal.cuh"
 
 namespace bfs {
 
-struct df {
-    float hi, lo;
+// A pair of double-float values: hi + lo for two sources.
+struct df2 {
+    f2 h, l;
 };
 
-__device__ __forceinline__ df mk(float h, float l) { return df{h, l}; }
-
-// |a| >= |b| (or a == 0)
-__device__ __forceinline__ df fast_two_sum(float a, float b)
+// a + b: Knuth's two-sum of the high parts, the error and the low parts added
+__device__ __forceinline__ df2 d2_add(df2 a, df2 b)
 {
-    float s = a + b;
-    return mk(s, b - (s - a));
+    const f2 s = f2_add(a.h, b.h);
+    const f2 bb = f2_sub(s, a.h);
+    const f2 e = f2_add(f2_sub(a.h, f2_sub(s, bb)), f2_sub(b.h, bb));
+    return df2{s, f2_add(e, f2_add(a.l, b.l))};
 }
 
-__device__ __forceinline__ df df_add(df a, df b)
+__device__ __forceinline__ df2 d2_sub(df2 a, df2 b)
 {
-    float s = a.hi + b.hi;
-    float bb = s - a.hi;
-    float e = (a.hi - (s - bb)) + (b.hi - bb);
-    e += a.lo + b.lo;
-    return fast_two_sum(s, e);
+    const f2 s = f2_sub(a.h, b.h);
+    const f2 bb = f2_sub(s, a.h);
+    const f2 e = f2_sub(f2_sub(a.h, f2_sub(s, bb)), f2_add(b.h, bb));
+    return df2{s, f2_add(e, f2_sub(a.l, b.l))};
 }
 
-__device__ __forceinline__ df df_neg(df a) { return mk(-a.hi, -a.lo); }
-__device__ __forceinline__ df df_sub(df a, df b) { return df_add(a, df_neg(b)); }
-
-__device__ __forceinline__ df df_add_f(df a, float b)
+// a b: two-product of the high parts, the cross terms added
+__device__ __forceinline__ df2 d2_mul(df2 a, df2 b)
 {
-    float s = a.hi + b;
-    float bb = s - a.hi;
-    float e = (a.hi - (s - bb)) + (b - bb);
-    e += a.lo;
-    return fast_two_sum(s, e);
+    const f2 p = f2_mul(a.h, b.h);
+    f2 e = f2_fma(a.h, b.h, f2_neg(p));
+    e = f2_fma(a.h, b.l, e);
+    return df2{p, f2_fma(a.l, b.h, e)};
 }
 
-__device__ __forceinline__ df df_mul(df a, df b)
+// x s + y t for float s, t
+__device__ __forceinline__ df2 d2_slope(df2 x, f2 s, df2 y, f2 t)
 {
-    float p = a.hi * b.hi;
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, e);
-    e = fmaf(a.lo, b.hi, e);
-    return fast_two_sum(p, e);
+    const f2 p = f2_mul(x.h, s), q = f2_mul(y.h, t);
+    f2 e = f2_fma(x.l, s, f2_fma(x.h, s, f2_neg(p)));
+    e = f2_add(e, f2_fma(y.l, t, f2_fma(y.h, t, f2_neg(q))));
+    const f2 v = f2_add(p, q);
+    const f2 bb = f2_sub(v, p);
+    const f2 r = f2_add(f2_sub(p, f2_sub(v, bb)), f2_sub(q, bb));
+    return df2{v, f2_add(r, e)};
 }
 
-__device__ __forceinline__ df df_mulf(df a, float b)
+// a = s^2 + t^2 + d^2.  SQ: rho2 is an exact multiple of 1/4, so rho2 - a.h is
+// exact (Sterbenz's lemma while d^2 <= rho2; beyond that both are multiples of
+// the spacing of a.h as long as a.h < 2^22) and one FMA gives the rest of d.h^2.
+template <bool SQ>
+__device__ __forceinline__ df2 d2_r2(df2 rho2, df2 d)
 {
-    float p = a.hi * b;
-    float e = fmaf(a.hi, b, -p);
-    e = fmaf(a.lo, b, e);
-    return fast_two_sum(p, e);
-}
-
-// The same three without the final renormalisation (the pair stays an exact
-// unevaluated sum, its low part up to about 2^-22 of the high one), for the
-// quantities of the pair sum that cannot cancel: sums of squares, powers of
-// 1/r, and products entering a renormalising accumulation.
-__device__ __forceinline__ df df_add_s(df a, df b)
-{
-    float s = a.hi + b.hi;
-    float bb = s - a.hi;
-    float e = (a.hi - (s - bb)) + (b.hi - bb);
-    e += a.lo + b.lo;
-    return mk(s, e);
-}
-
-__device__ __forceinline__ df df_mul_s(df a, df b)
-{
-    float p = a.hi * b.hi;
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, e);
-    e = fmaf(a.lo, b.hi, e);
-    return mk(p, e);
-}
-
-__device__ __forceinline__ df df_sqr_s(df a)
-{
-    float p = a.hi * a.hi;
-    float e = fmaf(a.hi, a.hi, -p);
-    e = fmaf(2.0f * a.hi, a.lo, e);
-    return mk(p, e);
-}
-
-__device__ __forceinline__ df df_sqr(df a)
-{
-    float p = a.hi * a.hi;
-    float e = fmaf(a.hi, a.hi, -p);
-    e = fmaf(2.0f * a.hi, a.lo, e);
-    return fast_two_sum(p, e);
-}
-
-// 1/sqrt(a): single-precision seed, one Newton step carried in double-float
-// (the step's residual 1 - a y0^2 is formed from the exact square of y0).
-__device__ __forceinline__ df df_rsqrt(df a)
-{
-    const float y0 = rsqrtf(a.hi);
-    const float p = y0 * y0;
-    const df y2 = mk(p, fmaf(y0, y0, -p));
-    const df q = df_mul(a, y2);
-    const float e = (1.0f - q.hi) - q.lo;
-    return mk(y0, 0.5f * y0 * e);
-}
-
-__device__ __forceinline__ df ld2(const float *p) { return mk(p[0], p[1]); }
-
-// Double-float source and target records (32 floats each):
-// source: 0 column, 1 row (mesh units, exact), then hi/lo pairs of
-//   2 zeta/dx  4 (beta+1)/dx  6 zeta_x  8 zeta_y dy/dx  10 beta_x  12 beta_y dy/dx
-//   14 w1 f  16 w2 zeta_x  18 w1 g  20 w2 sigma beta_x  22 w1  24 w2
-// target: 0 column, 1 row, then 2 zeta*/dx  4 zeta*/dx + 1/dx  6 (beta*+1)/dx - 1/dx
-//   8 (beta*+1)/dx  10 f*  12 g*  14 A  16 B dy/dx  18 C (dy/dx)^2
-constexpr int DREC = 32;
-
-__device__ __forceinline__ void split2(double v, float *o)
-{
-    float h = (float)v;
-    o[0] = h;
-    o[1] = (float)(v - (double)h);
-}
-
-__global__ void k_records_df(const double *__restrict__ src64, const double *__restrict__ tgt64,
-                             float *__restrict__ srcdf, float *__restrict__ tgtdf, int Ns_cap, int Nt,
-                             double ry)
-{
-    int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < Ns_cap) {
-        const double *r = src64 + (size_t)e * REC;
-        float *o = srcdf + (size_t)e * DREC;
-        o[0] = (float)r[0];
-        o[1] = (float)r[14];
-        split2(r[2], o + 2);
-        split2(r[3], o + 4);
-        split2(r[4], o + 6);
-        split2(r[5] * ry, o + 8);
-        split2(r[6], o + 10);
-        split2(r[7] * ry, o + 12);
-        split2(r[8], o + 14);
-        split2(r[9], o + 16);
-        split2(r[10], o + 18);
-        split2(r[11], o + 20);
-        split2(r[12], o + 22);
-        split2(r[13], o + 24);
-        for (int k = 26; k < DREC; k++) o[k] = 0.0f;
-        return;
+    if constexpr (SQ) {
+        const f2 a = f2_fma(d.h, d.h, rho2.h);
+        const f2 e = f2_fma(d.h, d.h, f2_sub(rho2.h, a));
+        return df2{a, f2_fma(f2_add(d.h, d.h), d.l, e)};
+    } else {
+        const f2 p = f2_mul(d.h, d.h);
+        const f2 e = f2_fma(f2_add(d.h, d.h), d.l, f2_fma(d.h, d.h, f2_neg(p)));
+        return d2_add(rho2, df2{p, e});
     }
-    e -= Ns_cap;
-    if (e >= Nt) return;
-    const double *t = tgt64 + (size_t)e * TREC;
-    float *o = tgtdf + (size_t)e * DREC;
-    o[0] = (float)t[0];
-    o[1] = (float)t[15];
-    split2(t[2], o + 2);
-    split2(t[11], o + 4);
-    split2(t[12], o + 6);
-    split2(t[3], o + 8);
-    split2(t[6], o + 10);
-    split2(t[7], o + 12);
-    split2(t[8], o + 14);
-    split2(t[9] * ry, o + 16);
-    split2(t[10] * ry * ry, o + 18);
-    for (int k = 20; k < DREC; k++) o[k] = 0.0f;
 }
+
+// The FP32 seed y0 of 1/sqrt(a), p + q = y0^2 exactly and m = a y0^2 - 1
+// (below 2^-21; the first FMA rounds a product within 2^-21 of 1 to about
+// 2^-46, the low parts follow).
+struct Seed {
+    f2 y, p, q, m;
+};
+
+__device__ __forceinline__ Seed d2_seed(df2 a)
+{
+    Seed s;
+    s.y = f2_rsq(a.h);
+    s.p = f2_mul(s.y, s.y);
+    s.q = f2_fma(s.y, s.y, f2_neg(s.p));
+    s.m = f2_fma(a.h, s.p, f2_both(-1.f));
+    s.m = f2_fma(a.h, s.q, s.m);
+    s.m = f2_fma(a.l, s.p, s.m);
+    return s;
+}
+
+// 1/sqrt(a) and 1/a from the seed
+__device__ __forceinline__ df2 d2_inv_r(const Seed &s)
+{
+    return df2{s.y, f2_mul(f2_mul(s.y, s.m), f2_fma(s.m, f2_both(0.375f), f2_both(-0.5f)))};
+}
+
+__device__ __forceinline__ df2 d2_inv_r2(const Seed &s)
+{
+    return df2{s.p, f2_fma(f2_mul(s.p, s.m), f2_add(s.m, f2_both(-1.f)), s.q)};
+}
+
+// the low part back within half a unit of the high one (|h| >= |l|)
+__device__ __forceinline__ df2 d2_norm(df2 a)
+{
+    const f2 s = f2_add(a.h, a.l);
+    return df2{s, f2_sub(a.l, f2_sub(s, a.h))};
+}
+
+__device__ __forceinline__ df2 both2(const float *p) { return df2{f2_both(p[0]), f2_both(p[1])}; }
 
 constexpr int PDF_TPB = 128, PDF_CH = 64;
 
-__global__ void __launch_bounds__(PDF_TPB)
+// Records: source pairs interleaved (value v of sources 2i and 2i+1 side by
+// side), see DSRC in bfs_internal.cuh; targets DTGT floats each.
+template <bool SQ>
+__global__ void __launch_bounds__(PDF_TPB, 4)
 k_pairs_df(const float *__restrict__ src, int per_split, const float *__restrict__ tgt, int Nt,
-           double *__restrict__ part, df ry, df ry2)
+           double *__restrict__ part, float ry2h, float ry2l, double ry, double dy)
 {
-    __shared__ __align__(16) float sh[PDF_CH * DREC];
+    __shared__ __align__(16) float sh[PDF_CH * DSRC];
     const int split = blockIdx.y;
-    const float *sb = src + (size_t)split * per_split * DREC;
+    const float *sb = src + (size_t)split * per_split * DSRC;
     const int t = blockIdx.x * PDF_TPB + threadIdx.x;
-    const float *tr = tgt + (size_t)min(t, Nt - 1) * DREC;
-    const float tx = tr[0], ty = tr[1];
-    const df tz = ld2(tr + 2), cTB = ld2(tr + 4), cBT = ld2(tr + 6), tB = ld2(tr + 8);
-    const df tf = ld2(tr + 10), tg = ld2(tr + 12), A = ld2(tr + 14), Bry = ld2(tr + 16),
-             Cry2 = ld2(tr + 18);
-    df aT1 = mk(0, 0), aT2 = mk(0, 0), aS = mk(0, 0), aB1 = mk(0, 0), aB2 = mk(0, 0);
+    const float *tr = tgt + (size_t)min(t, Nt - 1) * DTGT;
+    const f2 tx = f2_both(tr[0]), ty = f2_both(tr[1]);
+    const df2 tz = both2(tr + 2), cTB = both2(tr + 4), cBT = both2(tr + 6), tB = both2(tr + 8);
+    const df2 ntf = df2{f2_both(-tr[10]), f2_both(-tr[11])}, ntg = df2{f2_both(-tr[12]), f2_both(-tr[13])};
+    const df2 tzx = both2(tr + 14), tzy = both2(tr + 16);
+    const df2 zero = df2{f2_both(0.f), f2_both(0.f)};
+    df2 aT = zero, aS = zero, aB = zero;
 
     for (int c0 = 0; c0 < per_split; c0 += PDF_CH) {
+        const int nc = min(PDF_CH, per_split - c0);
         __syncthreads();
-        const float4 *g = reinterpret_cast<const float4 *>(sb + (size_t)c0 * DREC);
+        const float4 *g = reinterpret_cast<const float4 *>(sb + (size_t)c0 * DSRC);
         float4 *sv = reinterpret_cast<float4 *>(sh);
-        for (int e = threadIdx.x; e < PDF_CH * DREC / 4; e += PDF_TPB) sv[e] = g[e];
+        for (int e = threadIdx.x; e < nc * DSRC / 4; e += PDF_TPB) sv[e] = g[e];
         __syncthreads();
-        for (int s = 0; s < PDF_CH; s++) {
-            const float *r = sh + s * DREC;
-            const float sx = r[0] - tx;  // exact: half-integer mesh offsets
-            const float dj = r[1] - ty;  // exact: integer row offset
-            const float sxx = sx * sx, djj = dj * dj, sdj = sx * dj;  // exact
-            const df rho2 = df_add_f(df_mulf(ry2, djj), sxx);
-            const df zs = ld2(r + 2), bs = ld2(r + 4), zxs = ld2(r + 6), zys = ld2(r + 8);
-            const df bxs = ld2(r + 10), bys = ld2(r + 12);
-            const df w1f = ld2(r + 14), w2zx = ld2(r + 16), w1g = ld2(r + 18), w2sb = ld2(r + 20);
-            const df w1 = ld2(r + 22), w2 = ld2(r + 24);
-            // S2 at the top target
-            {
-                const df q = df_add(df_add(df_mulf(A, sxx), df_mulf(Bry, sdj)), df_mulf(Cry2, djj));
-                aS = df_add(aS, df_mul_s(w2, df_rsqrt(q)));
+#pragma unroll 1
+        for (int i = 0; i < nc / 2; i++) {
+            const f2 *r = reinterpret_cast<const f2 *>(sh) + i * DSRC;
+            auto val = [&](int k) { return df2{r[k], r[k + 1]}; };
+            const f2 sx = f2_sub(r[0], tx);  // exact: half-integer mesh offsets
+            const f2 dj = f2_sub(r[1], ty);  // exact: integer row offset
+            df2 rho2;
+            if constexpr (SQ) {
+                rho2 = df2{f2_fma(dj, dj, f2_mul(sx, sx)), f2_both(0.f)};
+            } else {
+                const f2 sxx = f2_mul(sx, sx), djj = f2_mul(dj, dj);  // exact
+                rho2 = d2_add(d2_mul(df2{f2_both(ry2h), f2_both(ry2l)}, df2{djj, f2_both(0.f)}),
+                              df2{sxx, f2_both(0.f)});
             }
-            // top target, top source
+            const df2 zs = val(2), bs = val(4), w1f = val(14), w1g = val(16);
+            const f2 cw = r[22];
+            // w S2 at the top target: A s^2 + B s t + C t^2 = s^2 + t^2 + (zeta_x* s + zeta_y* t)^2
             {
-                const df d = df_sub(zs, tz);
-                const df ri = df_rsqrt(df_add_s(rho2, df_sqr_s(d)));
-                const df ri3 = df_mul_s(df_sqr_s(ri), ri);
-                const df num = df_sub(df_sub(d, df_mulf(zxs, sx)), df_mulf(zys, dj));
-                const df dens = df_sub(w1f, df_mul(tf, w1));
-                aT1 = df_add(aT1, df_mul_s(df_mul_s(dens, num), ri3));
-                aT2 = df_add(aT2, df_mul_s(w2zx, ri));
+                const df2 ri = d2_inv_r(d2_seed(d2_r2<SQ>(rho2, d2_slope(tzx, sx, tzy, dj))));
+                aS = d2_add(aS, df2{f2_mul(cw, ri.h), f2_mul(cw, ri.l)});
             }
-            // top target, bottom source
+            const df2 gt = d2_slope(val(6), sx, val(8), dj);
+            const df2 zxd = val(18);
+            // top target, top source: w (f - f*) K1 + w zeta_x K2
             {
-                const df d = df_sub(bs, cTB);
-                const df ri = df_rsqrt(df_add_s(rho2, df_sqr_s(d)));
-                const df ri3 = df_mul_s(df_sqr_s(ri), ri);
-                const df num = df_sub(df_sub(d, df_mulf(bxs, sx)), df_mulf(bys, dj));
-                aT1 = df_sub(aT1, df_mul_s(df_mul_s(w1g, num), ri3));
-                aT2 = df_add(aT2, df_mul_s(w2sb, ri));
+                const df2 d = d2_sub(zs, tz);
+                const Seed s = d2_seed(d2_r2<SQ>(rho2, d));
+                // w f - w f*: w is a power of two, so the product is exact
+                const f2 v = f2_fma(ntf.h, cw, w1f.h);
+                const f2 bb = f2_sub(v, w1f.h);
+                const f2 e = f2_add(f2_sub(w1f.h, f2_sub(v, bb)), f2_fma(ntf.h, cw, f2_neg(bb)));
+                const df2 dens = df2{v, f2_add(e, f2_fma(ntf.l, cw, w1f.l))};
+                const df2 u = d2_add(d2_mul(d2_mul(dens, d2_sub(d, gt)), d2_inv_r2(s)), zxd);
+                aT = d2_add(aT, d2_mul(u, d2_inv_r(s)));
             }
-            // bottom target, top source
+            // bottom target, top source: w f K1 + w zeta_x K2
             {
-                const df d = df_sub(zs, cBT);
-                const df ri = df_rsqrt(df_add_s(rho2, df_sqr_s(d)));
-                const df ri3 = df_mul_s(df_sqr_s(ri), ri);
-                const df num = df_sub(df_sub(d, df_mulf(zxs, sx)), df_mulf(zys, dj));
-                aB1 = df_add(aB1, df_mul_s(df_mul_s(w1f, num), ri3));
-                aB2 = df_add(aB2, df_mul_s(w2zx, ri));
+                const df2 d = d2_sub(zs, cBT);
+                const Seed s = d2_seed(d2_r2<SQ>(rho2, d));
+                const df2 u = d2_add(d2_mul(d2_mul(w1f, d2_sub(d, gt)), d2_inv_r2(s)), zxd);
+                aB = d2_add(aB, d2_mul(u, d2_inv_r(s)));
             }
-            // bottom target, bottom source
+            const df2 gb = d2_slope(val(10), sx, val(12), dj);
+            // top target, bottom source: -w g K1(beta) + w sigma beta_x K2(beta)
             {
-                const df d = df_sub(bs, tB);
-                const df ri = df_rsqrt(df_add_s(rho2, df_sqr_s(d)));
-                const df ri3 = df_mul_s(df_sqr_s(ri), ri);
-                const df num = df_sub(df_sub(d, df_mulf(bxs, sx)), df_mulf(bys, dj));
-                const df dens = df_sub(w1g, df_mul(tg, w1));
-                aB1 = df_sub(aB1, df_mul_s(df_mul_s(dens, num), ri3));
+                const df2 d = d2_sub(bs, cTB);
+                const Seed s = d2_seed(d2_r2<SQ>(rho2, d));
+                const df2 u = d2_add(d2_mul(d2_mul(w1g, d2_sub(gb, d)), d2_inv_r2(s)), val(20));
+                aT = d2_add(aT, d2_mul(u, d2_inv_r(s)));
+            }
+            // bottom target, bottom source: -w (g - g*) K1(beta)
+            {
+                const df2 d = d2_sub(bs, tB);
+                const Seed s = d2_seed(d2_r2<SQ>(rho2, d));
+                const f2 v = f2_fma(ntg.h, cw, w1g.h);
+                const f2 bb = f2_sub(v, w1g.h);
+                const f2 e = f2_add(f2_sub(w1g.h, f2_sub(v, bb)), f2_fma(ntg.h, cw, f2_neg(bb)));
+                const df2 dens = df2{v, f2_add(e, f2_fma(ntg.l, cw, w1g.l))};
+                aB = d2_add(aB, d2_mul(d2_mul(d2_mul(dens, d2_sub(gb, d)), d2_inv_r2(s)), d2_inv_r(s)));
+            }
+            if ((i & 3) == 3) {  // the low parts collect one rounding error per term
+                aT = d2_norm(aT);
+                aS = d2_norm(aS);
+                aB = d2_norm(aB);
             }
         }
     }
     if (t >= Nt) return;
-    const df acc[NACC] = {df_add(aT1, aT2), aS, df_add(aB1, aB2)};
+    // the two sources' halves joined in FP64, times the factor left out of the weights
+    const df2 acc[NACC] = {aT, aS, aB};
 #pragma unroll
-    for (int q = 0; q < NACC; q++)
-        part[((size_t)split * NACC + q) * Nt + t] = (double)acc[q].hi + (double)acc[q].lo;
+    for (int q = 0; q < NACC; q++) {
+        float h0, h1, l0, l1;
+        f2_unpack(acc[q].h, h0, h1);
+        f2_unpack(acc[q].l, l0, l1);
+        const double v = ((double)h0 + (double)h1) + (double)(l0 + l1);
+        part[((size_t)split * NACC + q) * Nt + t] = v * (q == 1 ? dy : ry);
+    }
 }
 
 PairPlan plan_df(int Nt, int Ns, int splits_req, int sms)
 {
-    return make_plan(Nt, Ns, PDF_TPB, 1, PDF_CH, splits_req, sms);
+    return fine_plan(Nt, Ns, PDF_TPB, 8, 5, splits_req, sms);
 }
 
 int pairs_df_launch(bfs_ctx *c, cudaStream_t s)
 {
-    const int tot = c->Ns_cap + c->Nt;
-    k_records_df<<<(tot + 255) / 256, 256, 0, s>>>(c->d_src64, c->d_tgt64, c->d_srcdf, c->d_tgtdf,
-                                                   c->Ns_cap, c->Nt, c->dy / c->dx);
-    c->launches++;
     const double ryd = c->dy / c->dx, ry2d = ryd * ryd;
-    df ry, ry2;
-    ry.hi = (float)ryd;
-    ry.lo = (float)(ryd - (double)ry.hi);
-    ry2.hi = (float)ry2d;
-    ry2.lo = (float)(ry2d - (double)ry2.hi);
+    const float ry2h = (float)ry2d, ry2l = (float)(ry2d - (double)ry2h);
     const PairPlan &p = c->plandf;
-    k_pairs_df<<<dim3(p.tiles, p.splits), PDF_TPB, 0, s>>>(c->d_srcdf, p.per_split, c->d_tgtdf, c->Nt,
-                                                          c->d_part, ry, ry2);
+    const dim3 grid(p.tiles, p.splits);
+    // the exact-square form needs s^2 + t^2 and the depth within its exact range (d2_r2)
+    const bool sq = c->dx == c->dy && c->N <= 1024 && c->M <= 512 && c->dx * 1024.0 >= 1.0;
+    if (sq)
+        k_pairs_df<true><<<grid, PDF_TPB, 0, s>>>(c->d_srcdf, p.per_split, c->d_tgtdf, c->Nt, c->d_part, ry2h,
+                                                  ry2l, ryd, c->dy);
+    else
+        k_pairs_df<false><<<grid, PDF_TPB, 0, s>>>(c->d_srcdf, p.per_split, c->d_tgtdf, c->Nt, c->d_part, ry2h,
+                                                   ry2l, ryd, c->dy);
     c->launches++;
     BFS_CUDA_TRY(c, cudaGetLastError());
     return BFS_OK;

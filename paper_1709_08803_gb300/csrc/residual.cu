@@ -70,16 +70,27 @@ __device__ __forceinline__ double ydiff(const double *q, int N, int M, int half,
 
 struct RecArgs {
     int N, M, half, Ns, Ns_cap, Nt;
-    int w64, w32;  // which source-record copies to write (a residual reads one)
+    int w64, w32, wdf;  // which record copies to write (a residual reads one)
     double x1, y1, dx, dy, sigma, jc, ry;
     double idx, i2dy;  // 1 / dx, 1 / (2 dy)
 };
 
-// Builds source records [0, Ns_cap) and target records [0, Nt) in FP64 and FP32.
-__global__ void k_records(double *nodal, const double *__restrict__ beta,
-                          const double *__restrict__ bx, const double *__restrict__ by,
-                          double *__restrict__ src64, float *__restrict__ src32,
-                          double *__restrict__ tgt64, float *__restrict__ tgt32, RecArgs a)
+// hi + lo float pair of v
+__device__ __forceinline__ void split2(double v, float &h, float &l)
+{
+    h = (float)v;
+    l = (float)(v - (double)h);
+}
+
+// Builds source records [0, Ns_cap) and target records [0, Nt) in the
+// arithmetics asked for.  Bound by the latency of the FP64 pipe (two
+// operations per clock and SM), so the CTAs are small, to spread over all SMs.
+constexpr int REC_TPB = 64;
+__global__ void __launch_bounds__(REC_TPB)
+k_records(double *nodal, const double *__restrict__ beta, const double *__restrict__ bx,
+          const double *__restrict__ by, double *__restrict__ src64, float *__restrict__ src32,
+          float *__restrict__ srcdf, double *__restrict__ tgt64, float *__restrict__ tgt32,
+          float *__restrict__ tgtdf, RecArgs a)
 {
     int e = blockIdx.x * blockDim.x + threadIdx.x;
     const int N = a.N, M = a.M;
@@ -88,6 +99,7 @@ __global__ void k_records(double *nodal, const double *__restrict__ beta,
     const double *ps = nodal + 6 * NM;
     double r[REC];
     if (e < a.Ns_cap) {
+        double c = 0.0, f = 0.0, g = 0.0;  // c: the trapezoid weight without dx dy
         if (e < a.Ns) {
             int img = e >= (int)NM;
             int i, j;
@@ -102,10 +114,12 @@ __global__ void k_records(double *nodal, const double *__restrict__ beta,
             double x = a.x1 + i * a.dx;
             double cx = (i == 0 || i == N - 1) ? 0.5 : 1.0;
             double cy = a.half ? ((j == M - 1) ? 0.5 : 1.0) : ((j == 0 || j == M - 1) ? 0.5 : 1.0);
-            double w = a.dx * a.dy * cx * cy;
+            c = cx * cy;
+            double w = a.dx * a.dy * c;
             double w1 = w * a.idx * a.idx, w2 = w * a.idx;
             double ysg = img ? -1.0 : 1.0;
-            double f = ph[q] - x, g = ps[q] - x;
+            f = ph[q] - x;
+            g = ps[q] - x;
             r[0] = (double)i - 0.5 * (N - 1);
             r[1] = (ysg * j - a.jc) * a.ry;
             r[2] = z[q] * a.idx;
@@ -131,6 +145,18 @@ __global__ void k_records(double *nodal, const double *__restrict__ beta,
         if (a.w32) {  // sources in interleaved pairs for the packed FP32x2 pair kernel
             float *d = src32 + (size_t)(e >> 1) * REC * 2 + (e & 1);
             for (int k = 0; k < REC; k++) d[2 * k] = k == 10 ? -(float)r[k] : (float)r[k];
+        }
+        if (a.wdf) {  // interleaved pairs; padding is far away with zero weight
+            float *d = srcdf + (size_t)(e >> 1) * DSRC * 2 + (e & 1);
+            const double cd = c * a.dx;
+            const double v[10] = {r[2], r[3], r[4], r[5] * a.ry, r[6], r[7] * a.ry,
+                                  c * f, c * g, cd * r[4], cd * a.sigma * r[6]};
+            d[0] = (float)r[0];
+            d[2] = (float)r[14];
+#pragma unroll
+            for (int k = 0; k < 10; k++) split2(v[k], d[2 * (2 + 2 * k)], d[2 * (3 + 2 * k)]);
+            d[44] = (float)c;
+            d[46] = 0.f;
         }
         return;
     }
@@ -163,9 +189,16 @@ __global__ void k_records(double *nodal, const double *__restrict__ beta,
     r[13] = pxs;
     r[14] = pys;
     r[15] = (double)l - a.jc;  // row coordinate in mesh units (exact)
-    for (int q = 0; q < TREC; q++) {
-        tgt64[(size_t)e * TREC + q] = r[q];
-        tgt32[(size_t)e * TREC + q] = (float)r[q];
+    for (int q = 0; q < TREC; q++) tgt64[(size_t)e * TREC + q] = r[q];
+    if (a.w32)
+        for (int q = 0; q < TREC; q++) tgt32[(size_t)e * TREC + q] = (float)r[q];
+    if (a.wdf) {
+        float *o = tgtdf + (size_t)e * DTGT;
+        const double v[8] = {r[2], r[11], r[12], r[3], r[6], r[7], r[4], r[5] * a.ry};
+        o[0] = (float)r[0];
+        o[1] = (float)r[15];
+#pragma unroll
+        for (int k = 0; k < 8; k++) split2(v[k], o[2 + 2 * k], o[3 + 2 * k]);
     }
 }
 
@@ -320,44 +353,6 @@ __device__ __forceinline__ void pair_tile(const double *__restrict__ src, int pe
 // pair_tile<float>: each half accumulates its sources over a chunk, the halves
 // are added and the chunk total enters the two-sum accumulator.
 // ---------------------------------------------------------------------------
-struct f2 {
-    unsigned long long v;
-};
-__device__ __forceinline__ f2 f2_pack(float a, float b)
-{
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void f2_unpack(f2 x, float &a, float &b)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
-}
-__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c)
-{
-    f2 d;
-    asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(d.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-    return d;
-}
-__device__ __forceinline__ f2 f2_mul(f2 a, f2 b)
-{
-    f2 d;
-    asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
-    return d;
-}
-__device__ __forceinline__ f2 f2_sub(f2 a, f2 b)
-{
-    f2 d;
-    asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
-    return d;
-}
-__device__ __forceinline__ f2 f2_rsq(f2 x)
-{
-    float a, b;
-    f2_unpack(x, a, b);
-    return f2_pack(rsqrtf(a), rsqrtf(b));
-}
-
 // Two shared-memory chunk buffers filled by 1-D bulk copies (cp.async.bulk,
 // completion counted in bytes on an mbarrier per buffer): the copy of the
 // next chunk is in flight while the CTA works on the current one.  `seq`
@@ -810,6 +805,7 @@ static RecArgs rec_args(const bfs_ctx *c)
     a.idx = 1.0 / c->dx;
     a.i2dy = 1.0 / (2.0 * c->dy);
     a.w64 = a.w32 = 1;
+    a.wdf = 0;
     return a;
 }
 
@@ -874,9 +870,11 @@ int unpack_launch(bfs_ctx *c, const double *u, cudaStream_t s, int which)
     RecArgs ra = rec_args(c);
     ra.w64 = which & 1;
     ra.w32 = (which >> 1) & 1;
+    ra.wdf = (which >> 2) & 1;
     int tot = c->Ns_cap + c->Nt;
-    k_records<<<(tot + 255) / 256, 256, 0, s>>>(c->d_nodal, c->d_beta, c->d_bx, c->d_by, c->d_src64,
-                                                 c->d_src32, c->d_tgt64, c->d_tgt32, ra);
+    k_records<<<(tot + REC_TPB - 1) / REC_TPB, REC_TPB, 0, s>>>(c->d_nodal, c->d_beta, c->d_bx, c->d_by, c->d_src64,
+                                                                c->d_src32, c->d_srcdf, c->d_tgt64, c->d_tgt32,
+                                                                c->d_tgtdf, ra);
     c->launches++;
     BFS_CUDA_TRY(c, cudaGetLastError());
     return BFS_OK;
@@ -889,7 +887,7 @@ constexpr int P32_TPB = 128, P32_TPT = 2, P32_CH = 128;
 int residual_launch(bfs_ctx *c, const double *u, double *Fu, int precision, cudaStream_t s)
 {
     // FP32C pairs read the FP32 source records, FP64 and double-float ones the FP64 records
-    int rc = unpack_launch(c, u, s, precision == BFS_FP32C ? 2 : 1);
+    int rc = unpack_launch(c, u, s, precision == BFS_FP32C ? 2 : (precision == BFS_DF64 ? 4 : 1));
     if (rc) return rc;
     const PairPlan &p = precision == BFS_FP32C ? c->plan32 : (precision == BFS_DF64 ? c->plandf : c->plan64);
     dim3 grid(p.tiles, p.splits);
