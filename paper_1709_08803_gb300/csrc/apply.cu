@@ -50,17 +50,20 @@ namespace bfs {
 
 struct FlowArgs {
     const float *pc;               // FP32 factors: block (k, m) row r at ((k nd + m - k + h) nb + r) ldp
-    const double *r;               // right-hand side, order of u
-    double *z;                     // result, order of u (may equal r)
+    const double *r;               // right-hand side, order of u (condensed blocks: slice by slice)
+    double *z;                     // result, in the same order
     unsigned long long *X, *Y;     // tagged slice-ordered vectors, M * nb each
     int nb, NB, M, h;
     int ldp;                       // padded row length of the FP32 factors (multiple of 4)
     int nslot;                     // shared-memory ring depth (task-table kernel)
+    int sw, vs;                    // words a CTA owns in a vector slice, and a slice has (task-table kernel)
+    int zpair;                     // write z as float pairs (condensed blocks; task-table kernel)
+    int rows;                      // rows of a slice per CTA at most: its compute warps (task-table kernel)
     unsigned int *tagp;            // device word: tag of this launch's first step; step (task) s
                                    // writes tag0 + s, and block 0 advances the word by ntags on exit
     int *flag;
     unsigned int spin;             // polls of one wait before giving up
-    const SweepTask *tasks;        // task table: group 0's tasks, then group 1's
+    const SweepDev *tasks;         // task table: group 0's tasks, then group 1's
     int ntask0, ntask1;            // tasks per group
     int G0;                        // CTAs of group 0 (the rest form group 1)
     int ntags;                     // tags one launch uses (= ntask0 + ntask1)
@@ -99,6 +102,42 @@ __device__ __forceinline__ void advance_tag(unsigned int *p, unsigned int tag0, 
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(next) : "memory");
 }
 
+// hi + lo += b: Knuth's two-sum (the explicit _rn operations keep the compiler
+// from contracting).  The sweeps' rows cancel, so their sums are carried as
+// pairs: the error left is that of the FP32 factors and products.
+__device__ __forceinline__ void pair_add(float &hi, float &lo, float b)
+{
+    const float s = __fadd_rn(hi, b);
+    const float bb = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
+    hi = s;
+}
+
+// Values of CPT tagged entries (those with cv set) once their tags are `tag`,
+// w holding what an earlier load returned; all entries still missing are polled
+// together, so that a wait costs one round trip through L2 whatever CPT is.
+// False after `spin` polls.
+template <int CPT>
+__device__ __forceinline__ bool await_words(const unsigned long long *p, const int (&col)[CPT], const bool (&cv)[CPT],
+                                            unsigned int tag, unsigned long long (&w)[CPT], float (&v)[CPT],
+                                            unsigned int spin)
+{
+    unsigned int spins = 0;
+    while (true) {
+        bool all = true;
+#pragma unroll
+        for (int q = 0; q < CPT; q++) all = all && (!cv[q] || (unsigned int)(w[q] >> 32) == tag);
+        if (all) break;
+        if (++spins > spin) return false;
+#pragma unroll
+        for (int q = 0; q < CPT; q++)
+            if (cv[q] && (unsigned int)(w[q] >> 32) != tag) w[q] = ld_word(p + col[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < CPT; q++) v[q] = cv[q] ? __uint_as_float((unsigned int)w[q]) : 0.f;
+    return true;
+}
+
 // Value of a tagged entry once its tag is `tag`; false after `spin` polls.
 __device__ __forceinline__ bool await_word(const unsigned long long *p, unsigned int tag, float &v,
                                            unsigned int spin)
@@ -114,10 +153,19 @@ __device__ __forceinline__ bool await_word(const unsigned long long *p, unsigned
     return true;
 }
 
-template <int RPC, int CPT>
+// Sums as float pairs for condensed blocks (whose rows cancel more), plain FP32
+// ones otherwise.
+template <bool PAIR>
+__device__ __forceinline__ void flow_add(float &hi, float &lo, float b)
+{
+    if constexpr (PAIR) pair_add(hi, lo, b);
+    else hi += b;
+}
+
+template <int RPC, int CPT, bool PAIR>
 __global__ void __launch_bounds__(FL_TPB, 1) k_apply_flow(FlowArgs a)
 {
-    __shared__ float red[RPC][FL_WARPS];
+    __shared__ float2 red[RPC][FL_WARPS];
     __shared__ unsigned int tag_sh;
     const float *pc = a.pc;
     const int nb = a.nb, NB = a.NB, M = a.M, h = a.h, nd = 2 * h + 1, G = gridDim.x;
@@ -199,9 +247,9 @@ __global__ void __launch_bounds__(FL_TPB, 1) k_apply_flow(FlowArgs a)
         int pass, k, lo, hi, crit;
         step_of(s, pass, k, lo, hi, crit);
         prefetch(s + 2);
-        float acc[RPC];
+        float acc[RPC], alo[RPC];
 #pragma unroll
-        for (int j = 0; j < RPC; j++) acc[j] = 0.f;
+        for (int j = 0; j < RPC; j++) acc[j] = alo[j] = 0.f;
         double xk = 0.0;
         if (pass == 0 && my_rv) xk = a.r[my_e + (size_t)k * NB];
 
@@ -240,7 +288,7 @@ __global__ void __launch_bounds__(FL_TPB, 1) k_apply_flow(FlowArgs a)
                     float t = 0.f;
 #pragma unroll
                     for (int q = 0; q < CPT; q++) t = fmaf(f[bb][j][q], v[bb][q], t);
-                    acc[j] = fmaf(sg, t, acc[j]);
+                    flow_add<PAIR>(acc[j], alo[j], sg * t);
                 }
             }
             if (two) m = m2;
@@ -259,25 +307,31 @@ __global__ void __launch_bounds__(FL_TPB, 1) k_apply_flow(FlowArgs a)
             const unsigned long long *vp = vec(pass, k, crit);
             const unsigned int tg = tag0 + (unsigned int)(s - 1);
             float v[CPT];
+            unsigned long long wv[CPT];
 #pragma unroll
             for (int q = 0; q < CPT; q++) {
                 v[q] = 0.f;
-                if (ok && cv[q]) ok = await_word(vp + col[q], tg, v[q], a.spin);
+                wv[q] = cv[q] ? ld_word(vp + col[q]) : 0ull;
             }
+            if (ok) ok = await_words<CPT>(vp, col, cv, tg, wv, v, a.spin);
 #pragma unroll
             for (int j = 0; j < RPC; j++) {
                 float t = 0.f;
 #pragma unroll
                 for (int q = 0; q < CPT; q++) t = fmaf(cf[j][q], v[q], t);
-                acc[j] = fmaf(sg, t, acc[j]);
+                flow_add<PAIR>(acc[j], alo[j], sg * t);
             }
         }
 #pragma unroll
         for (int j = 0; j < RPC; j++) {
-            float t = acc[j];
+            float t = acc[j], tl = alo[j];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0) red[j][warp] = t;
+            for (int o = 16; o > 0; o >>= 1) {
+                const float ol = PAIR ? __shfl_xor_sync(0xffffffffu, tl, o) : 0.f;
+                flow_add<PAIR>(t, tl, __shfl_xor_sync(0xffffffffu, t, o));
+                tl += ol;
+            }
+            if (lane == 0) red[j][warp] = make_float2(t, tl);
         }
         if (!__syncthreads_and(ok)) {
             if (tid == 0) {
@@ -287,16 +341,21 @@ __global__ void __launch_bounds__(FL_TPB, 1) k_apply_flow(FlowArgs a)
             return;
         }
         if (my_rv) {
-            float t = 0.f;
+            float t = 0.f, tl = 0.f;
 #pragma unroll
-            for (int w = 0; w < FL_WARPS; w++) t += red[my_j][w];
+            for (int w = 0; w < FL_WARPS; w++) {
+                flow_add<PAIR>(t, tl, red[my_j][w].x);
+                tl += red[my_j][w].y;
+            }
             const size_t si = (size_t)k * nb + blockIdx.x + my_j * G;
             const unsigned int tg = tag0 + (unsigned int)s;
             if (pass == 0) {
-                st_word(a.Y + si, (float)(xk + (double)t), tg);
+                const float xh = (float)xk;
+                pair_add(t, tl, xh);
+                st_word(a.Y + si, t + (tl + (float)(xk - (double)xh)), tg);
             } else {
-                st_word(a.X + si, t, tg);
-                a.z[my_e + (size_t)k * NB] = (double)t;
+                st_word(a.X + si, t + tl, tg);
+                a.z[my_e + (size_t)k * NB] = (double)t + (double)tl;
             }
         }
         __syncthreads();  // red is rewritten by the next step
@@ -305,103 +364,110 @@ __global__ void __launch_bounds__(FL_TPB, 1) k_apply_flow(FlowArgs a)
 }
 
 // ---------------------------------------------------------------------------
-// Task-table kernel for slice blocks that fit its tiles (rows of a slice per
-// CTA <= RPC, nb <= CT CPT, at most SW_BMAX blocks per task).  Each CTA owns a
-// contiguous run of rows, so its rows of one block are one contiguous span of
-// the padded FP32 factors.  A producer warp streams the spans of every block
-// of a task into a ring of `nslot` shared-memory slots with 1-D bulk copies
-// (cp.async.bulk, completion counted in bytes on a "full" mbarrier per slot),
-// up to nslot - 1 tasks ahead; the compute warps release a slot on its "empty"
-// mbarrier once they have read it.  No compute thread spends issue slots or
-// load-queue entries on the factors.
+// Task-table kernel for slice blocks that fit its tiles (at most 8 rows of a
+// slice per CTA, at most 576 columns, at most SW_BMAX blocks per task).
+//
+// What bounds it is the latency of one task: the vector that the group's
+// previous task wrote has to reach every CTA through L2, be multiplied and be
+// written again, about M times in a row.  So the roles are split by warp, and
+// nothing but that vector's own path is on it:
+//   - a producer warp streams the CTA's rows of every block of a task into a ring
+//     of `nslot` shared-memory slots with 1-D bulk copies (cp.async.bulk,
+//     completion counted in bytes on a "full" mbarrier per slot), up to nslot - 1
+//     tasks ahead;
+//   - PW poll warps own two vector entries a thread and do nothing but load tagged
+//     words and put their values into shared memory: a task's prefetched vectors
+//     first ("early" mbarrier), then the critical one ("crit" mbarrier), both
+//     words polled in one loop without sleeping in between;
+//   - one compute warp per row: 16-byte shared loads of the row and the vectors, the
+//     terms that need not wait first, then the critical one, a shuffle reduction,
+//     and lane 0 writes the entry.  No barrier of the CTA is left in the loop.
+// The last two critical vectors stay in the compute warps' registers, where the
+// next tasks need them again, and the right-hand sides are staged at the start.
+//
+// 181 x 61 (h = 3, 62 dependent tasks), condensed blocks: 104 us a launch, 1.7 us
+// a task; the kernel before it (columns over threads, a CTA barrier and a
+// cross-warp sum per task) took 133 us on the same blocks and 139 us on the full
+// ones.  241 x 81 (h = 4): 0.99 ms (one-ended, k_apply_flow) -> 0.19 ms.
+//
+// Buffers: a poll warp writes for task s only once every compute warp is done
+// with task s - 2 (the ring's "empty" barriers), so a task's vectors alternate
+// between two sets.  Every wait is
+// bounded; a warp that gives up raises bit 2 of the flag and `dead`, which ends
+// the other warps' waits.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned int smem_u32(const void *p)
 {
     return (unsigned int)__cvta_generic_to_shared(p);
 }
 
-__device__ __forceinline__ bool mbar_wait(unsigned int bar, unsigned int parity, unsigned int spin)
+__device__ __forceinline__ bool mbar_try(unsigned int bar, unsigned int parity)
 {
-    for (unsigned int i = 0; i < spin; i++) {
-        unsigned int done;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (done) return true;
+    unsigned int done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return done != 0;
+}
+
+// Waits inside the CTA last as long as its poll warps' waits, whose polls are L2
+// round trips: SW_WAIT of these cheaper polls for each of theirs.
+constexpr unsigned long long SW_WAIT = 64;
+
+__device__ __forceinline__ bool mbar_wait(unsigned int bar, unsigned int parity, unsigned int spin, volatile int *dead)
+{
+    const unsigned long long lim = SW_WAIT * spin;
+    for (unsigned long long i = 0; i < lim; i++) {
+        if (mbar_try(bar, parity)) return true;
+        if (dead && *dead) return false;
     }
     return false;
 }
 
-// barrier 1 over the CT compute threads, AND of their predicates
-__device__ __forceinline__ bool compute_sync_and(bool pred, int ct)
+__device__ __forceinline__ void mbar_arrive(const void *bar)
 {
-    unsigned int r;
-    asm volatile(
-        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.and.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
-        : "=r"(r)
-        : "r"((unsigned int)pred), "r"(ct)
-        : "memory");
-    return r != 0;
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-// Sums v[j] (j < R, R a power of two <= 32) over the 32 lanes of a warp by a
-// reduce-scatter: each halving step trades half of the rows with the partner
-// lane, so R rows cost log2(R) + (R - 1) shuffles instead of 5 R.  Lane l ends
-// with the warp total of row `row`; the 32 / R lanes that share a row hold the
-// same total.
-template <int R>
-__device__ __forceinline__ float warp_rows_sum(const float (&acc)[R], int lane, int &row)
+__device__ __forceinline__ void mbar_init(const void *bar, unsigned int count)
 {
-    float v[R];
-#pragma unroll
-    for (int i = 0; i < R; i++) v[i] = acc[i];
-    int r = 0, off = 16;
-#pragma unroll
-    for (int n = R; n > 1; n >>= 1) {
-        const bool up = (lane & off) != 0;
-        const int hlf = n >> 1;
-#pragma unroll
-        for (int i = 0; i < hlf; i++) {
-            const float send = up ? v[i] : v[i + hlf];
-            const float keep = up ? v[i + hlf] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-        }
-        if (up) r += hlf;
-        off >>= 1;
-    }
-    for (; off >= 1; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
-    row = r;
-    return v[0];
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
 
-template <int CT, int RPC, int CPT>
-__global__ void __launch_bounds__(CT + 32, 1) k_apply_sweep(FlowArgs a)
+static_assert(SW_HW == 2, "the compute warps hold two critical vectors in registers");
+constexpr int SW_ROWS = 8;  // compute warps at most, one row each
+constexpr long long SW_BACKOFF = 400;
+
+template <int PW, int WPT, int NQ, int BM>
+__global__ void __launch_bounds__(32 * (SW_ROWS + PW + 1), 1) k_apply_sweep(FlowArgs a)
 {
-    constexpr int WARPS = CT / 32;
-    constexpr int BM = SW_BMAX;
-    constexpr int MAXSLOT = 8;
-    static_assert(32 % RPC == 0 && RPC * BM >= 1, "rows per CTA must divide the warp");
-    extern __shared__ __align__(128) float ring[];  // nslot x BM x RPC x ldp, then the group's tasks
-    __shared__ __align__(8) unsigned long long full[MAXSLOT], empty[MAXSLOT];
-    __shared__ float red[2][RPC][WARPS];
+    constexpr int MAXSLOT = 8, PT = 32 * PW;  // poll threads, each owning WPT words
+    static_assert(BM <= SW_BMAX, "task table rows");
+    extern __shared__ __align__(128) float ring[];  // nslot x (h + 1) x rows x ldp, vector buffers, the group's tasks
+    __shared__ __align__(8) unsigned long long full[MAXSLOT], empty[MAXSLOT], early[2], crit[2];
     __shared__ unsigned int tag_sh;
     __shared__ int abort_sh;
+    __shared__ volatile int dead;
+    __shared__ float outv[4][SW_ROWS];  // a task's rows, until the CTA's last warp stores them together
+    __shared__ int ndone;               // rows done since the launch
     const float *pc = a.pc;
     const int nb = a.nb, NB = a.NB, h = a.h, nd = 2 * h + 1, ldp = a.ldp;
-    const int nslot = a.nslot;
+    const int nslot = a.nslot, rows = a.rows;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const size_t slot_floats = (size_t)BM * RPC * ldp;
+    const size_t slot_floats = (size_t)(h + 1) * rows * ldp;
     // CTA group and its tasks
     const int grp = (int)blockIdx.x < a.G0 ? 0 : 1;
-    const int Gg = grp ? (int)gridDim.x - a.G0 : a.G0;
+    const int Gg = a.G0;  // CTAs of either group
     const int lb = grp ? (int)blockIdx.x - a.G0 : (int)blockIdx.x;
-    const SweepTask *gtasks = a.tasks + (grp ? a.ntask0 : 0);
+    const SweepDev *gtasks = a.tasks + (grp ? a.ntask0 : 0);
     const int ntask = grp ? a.ntask1 : a.ntask0;
+    float *vbuf = ring + (size_t)nslot * slot_floats;  // 2 critical vectors of ldp, then 2 x (h + 1) early ones
     // the task table, staged once: a descriptor read from global memory at
     // every step would put an L2 round trip in front of each step's waits
-    SweepTask *tasks = reinterpret_cast<SweepTask *>(ring + (size_t)nslot * slot_floats);
+    SweepDev *tasks = reinterpret_cast<SweepDev *>(vbuf + (size_t)(2 + 2 * (h + 1)) * ldp);
+    float2 *xs = reinterpret_cast<float2 *>(tasks + ntask);  // right-hand sides of this CTA's rows, task by task
     // rows [r0, r0 + nrv) of every slice: the first nb % Gg CTAs take one row more
     const int base = nb / Gg, extra = nb % Gg;
     const int nrv = base + (lb < extra ? 1 : 0);
@@ -411,23 +477,47 @@ __global__ void __launch_bounds__(CT + 32, 1) k_apply_sweep(FlowArgs a)
     if (tid == 0) {
         abort_sh = (ld_tag(reinterpret_cast<const unsigned int *>(a.flag)) & 2u) != 0;
         tag_sh = ld_tag(a.tagp);
+        dead = 0;
+        ndone = 0;
         for (int i = 0; i < nslot; i++) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&full[i])) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[i])) : "memory");
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], nrv);
+        }
+        for (int i = 0; i < 2; i++) {
+            mbar_init(&early[i], PW);
+            mbar_init(&crit[i], PW);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    for (int i = tid; i < (2 + 2 * (h + 1)) * ldp; i += blockDim.x) vbuf[i] = 0.f;  // the padding stays 0
+    for (int i = tid; i < ntask * rows; i += blockDim.x) {  // as float pairs; 0 for z tasks
+        const int s = i / rows, j = i - s * rows;
+        float2 x = make_float2(0.f, 0.f);
+        if (gtasks[s].head.y == 0 && j < nrv) {
+            const int row = r0 + j, g = row / NB, pp = row - g * NB;
+            const double xk = a.r[(size_t)g * NB * a.M + pp + (size_t)gtasks[s].head.x * NB];
+            x.x = (float)xk;
+            x.y = (float)(xk - (double)x.x);
+        }
+        xs[i] = x;
+    }
     {
-        const int *src = reinterpret_cast<const int *>(gtasks);
-        int *dst = reinterpret_cast<int *>(tasks);
-        const int words = ntask * (int)(sizeof(SweepTask) / sizeof(int));
+        const int4 *src = reinterpret_cast<const int4 *>(gtasks);
+        int4 *dst = reinterpret_cast<int4 *>(tasks);
+        const int words = ntask * (int)(sizeof(SweepDev) / sizeof(int4));
         for (int i = tid; i < words; i += blockDim.x) dst[i] = src[i];
     }
     __syncthreads();
     if (abort_sh) return;  // an earlier wait timed out: the host resets the vectors first
     const unsigned int tag0 = tag_sh;
+    auto give_up = [&]() {
+        if (lane == 0) {
+            dead = 1;
+            atomicOr(a.flag, 2);
+        }
+    };
 
-    if (warp == WARPS) {
+    if (warp == rows + PW) {
         // producer warp: the rows [r0, r0 + nrv) of every block of task q into slot q % nslot
         int q = 0;
         bool fine = true;
@@ -436,16 +526,15 @@ __global__ void __launch_bounds__(CT + 32, 1) k_apply_sweep(FlowArgs a)
             const int slot = q % nslot;
             if (q >= nslot) {
                 int w = 1;
-                if (lane == 0)
-                    w = mbar_wait(smem_u32(&empty[slot]), (unsigned int)((q / nslot - 1) & 1), a.spin) ? 1 : 0;
+                if (lane == 0) w = mbar_wait(smem_u32(&empty[slot]), (unsigned int)((q / nslot - 1) & 1), a.spin, &dead);
                 w = __shfl_sync(0xffffffffu, w, 0);
                 if (!w) {
-                    if (lane == 0) atomicOr(a.flag, 2);
+                    give_up();
                     fine = false;
                     break;
                 }
             }
-            const int k = tasks[q].k, nblk = tasks[q].nblk;
+            const int k = tasks[q].head.x, nblk = tasks[q].head.z;
             const unsigned int fb = smem_u32(&full[slot]);
             if (lane == 0) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -454,12 +543,11 @@ __global__ void __launch_bounds__(CT + 32, 1) k_apply_sweep(FlowArgs a)
                              : "memory");
             }
             __syncwarp();
-            for (int idx = lane; idx < nblk * RPC; idx += 32) {
-                const int p = idx / RPC, j = idx - p * RPC;
-                if (j >= nrv) continue;
-                const int m = tasks[q].m[p];
+            for (int idx = lane; idx < nblk * nrv; idx += 32) {
+                const int p = idx / nrv, j = idx - p * nrv;
+                const int m = tasks[q].blk[p].x;
                 const float *src = pc + (((size_t)k * nd + (m - k + h)) * nb + r0 + j) * ldp;
-                float *dst = ring + (size_t)slot * slot_floats + ((size_t)p * RPC + j) * ldp;
+                float *dst = ring + (size_t)slot * slot_floats + ((size_t)p * rows + j) * ldp;
                 asm volatile(
                     "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                         smem_u32(dst)),
@@ -471,162 +559,221 @@ __global__ void __launch_bounds__(CT + 32, 1) k_apply_sweep(FlowArgs a)
         if (lane == 0) {
             const int last = fine ? ntask - 1 : q - 1;
             for (int pq = max(0, last - nslot + 1); pq <= last; pq++)
-                if (!mbar_wait(smem_u32(&full[pq % nslot]), (unsigned int)((pq / nslot) & 1), a.spin)) break;
+                if (!mbar_wait(smem_u32(&full[pq % nslot]), (unsigned int)((pq / nslot) & 1), a.spin, nullptr)) break;
         }
         return;
     }
 
-    // compute warps: thread tid owns the columns tid + q CT of every block
-    int col[CPT];
-    bool cv[CPT];
+    if (warp >= rows) {
+        // poll warps: words pt, pt + PT, ... of every vector slice; word w holds row w mod sw
+        // of CTA w / sw
+        const int pt = tid - 32 * rows;
+        int col[WPT], dst[WPT];
+        bool cv[WPT];
 #pragma unroll
-    for (int q = 0; q < CPT; q++) {
-        col[q] = tid + q * CT;
-        cv[q] = col[q] < nb;
-        if (!cv[q]) col[q] = 0;
+        for (int q = 0; q < WPT; q++) {
+            col[q] = pt + q * PT;
+            const int c = col[q] / a.sw, j = col[q] - c * a.sw;
+            cv[q] = c < Gg && j < base + (c < extra ? 1 : 0);
+            dst[q] = c * base + min(c, extra) + j;
+        }
+        // task s: blocks [e0, e1) are early, block e1 is critical if there is one
+        auto early_range = [&](int4 hd, int &e0, int &e1) {
+            e0 = (hd.w & 1) + ((hd.w >> 1) & 1);
+            e1 = hd.z - ((hd.w >> 2) & 1);
+        };
+        int4 blk[BM], head = tasks[0].head;  // of the task at hand; its early words, loaded a task ahead
+        unsigned long long pre[BM][WPT], wc[WPT];
+        auto load = [&](int s) {
+            int e0, e1;
+            head = tasks[s].head;
+#pragma unroll
+            for (int p = 0; p < BM; p++) blk[p] = tasks[s].blk[p];
+            early_range(head, e0, e1);
+#pragma unroll
+            for (int p = 0; p < BM; p++)
+#pragma unroll
+                for (int q = 0; q < WPT; q++)
+                    pre[p][q] = (p >= e0 && p < e1 && cv[q]) ? ld_word(a.Y + blk[p].y + col[q]) : 0ull;
+        };
+        bool ok = true;
+        int sl = 0, sl1 = 0;              // ring slots of tasks s - 1 and s - 2
+        unsigned int pr = 0u, pr1 = 0u;   // and the parities of their empty barriers
+        load(0);
+        for (int s = 0; s < ntask; s++) {
+            int e0, e1;
+            early_range(head, e0, e1);
+            float v[WPT];
+            // the buffers of task s - 2 are free once every compute warp is done with it
+            if (s >= 2) ok = mbar_wait(smem_u32(&empty[sl1]), pr1, a.spin, &dead);
+#pragma unroll
+            for (int p = 0; p < BM; p++) {
+                if (p < e0 || p >= e1 || !ok) continue;
+                ok = await_words<WPT>(a.Y + blk[p].y, col, cv, tag0 + (unsigned int)blk[p].z, pre[p], v, a.spin);
+                float *e = vbuf + (size_t)(2 + (s & 1) * (h + 1) + p) * ldp;
+#pragma unroll
+                for (int q = 0; q < WPT; q++)
+                    if (cv[q]) e[dst[q]] = v[q];
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&early[s & 1]);
+            const bool has_crit = (head.w & 4) != 0;
+            int4 cb = blk[0];
+#pragma unroll
+            for (int p = 1; p < BM; p++)
+                if (p == e1) cb = blk[p];
+            if (s + 1 < ntask) load(s + 1);
+            // the critical vector is polled from SW_BACKOFF clocks after this CTA finished its
+            // own rows of it: polls before that rarely succeed, and CTAs polling the same few
+            // lines slow the stores that they wait for (181 x 61, whole apply: 165 us
+            // without the pause, 138 us with 400 clocks, 147 us with 800)
+            if (has_crit) {
+                const unsigned long long *cptr = a.Y + cb.y;
+                ok = ok && mbar_wait(smem_u32(&empty[sl]), pr, a.spin, &dead);
+                for (const long long c0 = clock64(); clock64() - c0 < SW_BACKOFF;) {}
+#pragma unroll
+                for (int q = 0; q < WPT; q++) wc[q] = cv[q] ? ld_word(cptr + col[q]) : 0ull;
+                if (ok) ok = await_words<WPT>(cptr, col, cv, tag0 + (unsigned int)cb.z, wc, v, a.spin);
+                float *e = vbuf + (size_t)(s & 1) * ldp;
+#pragma unroll
+                for (int q = 0; q < WPT; q++)
+                    if (cv[q]) e[dst[q]] = v[q];
+            }
+            if (!__all_sync(0xffffffffu, ok)) {
+                give_up();
+                return;
+            }
+            if (lane == 0) mbar_arrive(&crit[s & 1]);
+            sl1 = sl;
+            pr1 = pr;
+            if (s > 0 && ++sl == nslot) {
+                sl = 0;
+                pr ^= 1u;
+            }
+        }
+        return;
     }
-    const int my_j = tid < nrv ? tid : -1;  // the row this thread finishes
-    size_t my_e = 0;                        // its index in the order of u (+ k NB for slice k)
-    if (my_j >= 0) {
-        const int rw = r0 + my_j, g = rw / NB, pp = rw - g * NB;
+
+    // compute warps: row r0 + warp of every slice, columns 4 lane + 128 q
+    if (warp >= nrv) return;
+    const int row = r0 + warp;
+    size_t my_e;  // its index in the order of u (+ k NB for slice k)
+    {
+        const int g = row / NB, pp = row - g * NB;
         my_e = (size_t)g * NB * a.M + pp;
     }
-    auto dot = [&](const float *S, int p, const float (&v)[CPT], float (&acc)[RPC], float sg) {
+    bool cq[NQ];
 #pragma unroll
-        for (int j = 0; j < RPC; j++) {
-            float u = 0.f;
+    for (int q = 0; q < NQ; q++) cq[q] = 4 * lane + 128 * q < ldp;
+    float acc[NQ], alo[NQ];
+    // acc += +- S v: four products a partial sum, the partial sums added as pairs,
+    // NQ independent chains
+    auto dot = [&](const float4 (&f)[NQ], const float4 (&x)[NQ], int plus) {
+        const unsigned int neg = plus ? 0u : 0x80000000u;
 #pragma unroll
-            for (int q = 0; q < CPT; q++)
-                if (cv[q] && j < nrv) u = fmaf(S[((size_t)p * RPC + j) * ldp + col[q]], v[q], u);
-            acc[j] = fmaf(sg, u, acc[j]);
+        for (int q = 0; q < NQ; q++) {
+            const float u = fmaf(f[q].w, x[q].w, fmaf(f[q].z, x[q].z, fmaf(f[q].y, x[q].y, f[q].x * x[q].x)));
+            pair_add(acc[q], alo[q], __uint_as_float(__float_as_uint(u) ^ neg));
         }
     };
-    auto vec_ptr = [&](int vec, int m) { return ((vec & 1) ? a.X : a.Y) + (size_t)m * nb; };
-    // words of a task's prefetched blocks (SW_EARLY), loaded at the end of the step before
-    unsigned long long pre[BM][CPT];
-    auto prefetch = [&](int s) {
+    auto fetch = [&](const float *p, float4 (&f)[NQ]) {
 #pragma unroll
-        for (int p = 0; p < BM; p++) {
-            const bool use = s < ntask && p < tasks[s].nblk && ((tasks[s].vec[p] >> 2) & 3) == SW_EARLY;
-            const unsigned long long *vp = use ? vec_ptr(tasks[s].vec[p], tasks[s].m[p]) : a.Y;
-#pragma unroll
-            for (int q = 0; q < CPT; q++) pre[p][q] = (use && cv[q]) ? ld_word(vp + col[q]) : 0ull;
-        }
+        for (int q = 0; q < NQ; q++)
+            f[q] = cq[q] ? *reinterpret_cast<const float4 *>(p + 4 * lane + 128 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
     };
-    // this thread's columns of the last SW_HW vectors that were a task's critical one
-    float win[SW_HW][CPT];
+    float4 w0[NQ], w1[NQ];  // this lane's columns of the last two critical vectors
 #pragma unroll
-    for (int i = 0; i < SW_HW; i++)
-#pragma unroll
-        for (int q = 0; q < CPT; q++) win[i][q] = 0.f;
-
-    bool ok = true;
-    prefetch(0);
+    for (int q = 0; q < NQ; q++) w0[q] = w1[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    int slot = 0;
+    unsigned int par = 0;  // of full[slot]
     for (int s = 0; s < ntask; s++) {
-        const int k = tasks[s].k, nblk = tasks[s].nblk, out = tasks[s].out;
-        // the critical vector: its first poll goes out before anything else
-        int cp = -1;
+        const int4 head = tasks[s].head;
+        const int nblk = head.z, win = head.w & 3, plus = head.w >> 4;
+        const bool has_crit = (head.w & 4) != 0;
+        const float *sp = ring + (size_t)slot * slot_floats + (size_t)warp * ldp;
+        const size_t bs = (size_t)rows * ldp;
 #pragma unroll
-        for (int p = 0; p < BM; p++)
-            if (p < nblk && ((tasks[s].vec[p] >> 2) & 3) == SW_CRIT) cp = p;
-        const int cvec = cp >= 0 ? tasks[s].vec[cp] : 0;
-        const unsigned long long *cptr = vec_ptr(cvec, cp >= 0 ? tasks[s].m[cp] : 0);
-        const unsigned int ctag = tag0 + (unsigned int)(cp >= 0 ? tasks[s].uid[cp] : 0);
-        unsigned long long wc[CPT];
-#pragma unroll
-        for (int q = 0; q < CPT; q++) wc[q] = (cp >= 0 && cv[q]) ? ld_word(cptr + col[q]) : 0ull;
-        double xk = 0.0;
-        if (out == 0 && my_j >= 0) xk = a.r[my_e + (size_t)k * NB];
-        const int slot = s % nslot;
-        const float *S = ring + (size_t)slot * slot_floats;
-        ok = ok && mbar_wait(smem_u32(&full[slot]), (unsigned int)((s / nslot) & 1), a.spin);
-        float acc[RPC];
-#pragma unroll
-        for (int j = 0; j < RPC; j++) acc[j] = 0.f;
-        // terms whose vectors this thread holds or has prefetched
-#pragma unroll
-        for (int p = 0; p < BM; p++) {
-            if (p < nblk && ok) {
-                const int vec = tasks[s].vec[p], src = (vec >> 2) & 3;
-                const float sg = (vec & 2) ? 1.f : -1.f;
-                float v[CPT];
-                if (src == SW_WIN) {
-                    const int wi = (vec >> 4) & 3;
-#pragma unroll
-                    for (int q = 0; q < CPT; q++) {
-                        v[q] = win[0][q];
-#pragma unroll
-                        for (int i = 1; i < SW_HW; i++)
-                            if (wi == i) v[q] = win[i][q];
-                    }
-                    dot(S, p, v, acc, sg);
-                } else if (src == SW_EARLY) {
-                    const unsigned int tg = tag0 + (unsigned int)tasks[s].uid[p];
-                    const unsigned long long *vp = vec_ptr(vec, tasks[s].m[p]);
-#pragma unroll
-                    for (int q = 0; q < CPT; q++) {
-                        v[q] = 0.f;
-                        if (!cv[q]) continue;
-                        if ((unsigned int)(pre[p][q] >> 32) == tg) v[q] = __uint_as_float((unsigned int)pre[p][q]);
-                        else if (ok) ok = await_word(vp + col[q], tg, v[q], a.spin);
-                    }
-                    dot(S, p, v, acc, sg);
+        for (int q = 0; q < NQ; q++) acc[q] = alo[q] = 0.f;
+        if (lane == 0) {
+            const float2 x = xs[s * rows + warp];
+            acc[0] = x.x;
+            alo[0] = x.y;
+        }
+        bool ok = mbar_wait(smem_u32(&full[slot]), par, a.spin, &dead);
+        // the row's entries of the blocks in the register window and of the critical one
+        const int nw = (win & 1) + (win >> 1);
+        float4 f0[NQ], f1[NQ], fc[NQ];
+        if (ok) {
+            if (win & 1) fetch(sp, f0);
+            if (win & 2) fetch(sp + (win & 1) * bs, f1);
+            if (has_crit) fetch(sp + (nblk - 1) * bs, fc);
+            if (win & 1) dot(f0, w0, plus & 1);
+            if (win & 2) dot(f1, w1, (plus >> (win & 1)) & 1);
+            const int nfree = nblk - (has_crit ? 1 : 0);
+            if (nw < nfree) {
+                ok = mbar_wait(smem_u32(&early[s & 1]), (unsigned int)((s >> 1) & 1), a.spin, &dead);
+#pragma unroll 1
+                for (int p = nw; p < nfree && ok; p++) {
+                    fetch(sp + p * bs, f0);
+                    fetch(vbuf + (size_t)(2 + (s & 1) * (h + 1) + p) * ldp, f1);
+                    dot(f0, f1, (plus >> p) & 1);
                 }
             }
         }
         // the critical term last: the vector the group's previous task wrote
-        if (cp >= 0 && ok) {
-            float v[CPT];
-#pragma unroll
-            for (int q = 0; q < CPT; q++) {
-                v[q] = 0.f;
-                if (!cv[q]) continue;
-                if ((unsigned int)(wc[q] >> 32) == ctag) v[q] = __uint_as_float((unsigned int)wc[q]);
-                else if (ok) ok = await_word(cptr + col[q], ctag, v[q], a.spin);
-            }
-#pragma unroll
-            for (int p = 0; p < BM; p++)
-                if (p == cp) dot(S, p, v, acc, (cvec & 2) ? 1.f : -1.f);
-#pragma unroll
-            for (int q = 0; q < CPT; q++) {
-#pragma unroll
-                for (int i = SW_HW - 1; i > 0; i--) win[i][q] = win[i - 1][q];
-                win[0][q] = v[q];
-            }
+        ok = ok && mbar_wait(smem_u32(&crit[s & 1]), (unsigned int)((s >> 1) & 1), a.spin, &dead);
+        if (!__all_sync(0xffffffffu, ok)) {
+            give_up();
+            return;
         }
-        float(&rd)[RPC][WARPS] = red[s & 1];
-        {
-            int row;
-            const float t = warp_rows_sum<RPC>(acc, lane, row);
-            if ((lane & (32 / RPC - 1)) == 0) rd[row][warp] = t;
-        }
-        if (!compute_sync_and(ok, CT)) {
-            if (tid == 0) atomicOr(a.flag, 2);
-            return;  // the producer drains its copies and returns
-        }
-        if (tid == 0)  // every compute warp has read slot `slot`
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[slot])) : "memory");
-        if (my_j >= 0) {
-            float u = 0.f;
+        if (has_crit) {
 #pragma unroll
-            for (int q = 0; q < WARPS; q++) u += rd[my_j][q];
-            const size_t si = (size_t)k * nb + r0 + my_j;
-            const unsigned int tg = tag0 + (unsigned int)((grp ? a.ntask0 : 0) + s);
-            if (out == 0) {
-                st_word(a.Y + si, (float)(xk + (double)u), tg);
-            } else {
-                st_word(a.X + si, u, tg);
-                a.z[my_e + (size_t)k * NB] = (double)u;
+            for (int q = 0; q < NQ; q++) w1[q] = w0[q];
+            fetch(vbuf + (size_t)(s & 1) * ldp, w0);
+            dot(fc, w0, (plus >> (nblk - 1)) & 1);
+        }
+#pragma unroll
+        for (int q = 1; q < NQ; q++) {
+            pair_add(acc[0], alo[0], acc[q]);
+            alo[0] += alo[q];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float oh = __shfl_down_sync(0xffffffffu, acc[0], o), ol = __shfl_down_sync(0xffffffffu, alo[0], o);
+            pair_add(acc[0], alo[0], oh);
+            alo[0] += ol;
+        }
+        // the CTA's rows go out in one store of its last warp: lines that many CTAs are
+        // about to poll are written once per CTA, not once per row
+        int last = 0;
+        if (lane == 0) {
+            outv[s & 3][warp] = acc[0] + alo[0];
+            __threadfence_block();
+            last = atomicAdd(&ndone, 1) == nrv * (s + 1) - 1;
+            mbar_arrive(&empty[slot]);  // every lane's reads of the slot came before the shuffles
+        }
+        if (__shfl_sync(0xffffffffu, last, 0)) {
+            __threadfence_block();
+            if (lane < nrv) {
+                const unsigned int tg = tag0 + (unsigned int)((grp ? a.ntask0 : 0) + s);
+                st_word((head.y ? a.X : a.Y) + (size_t)head.x * a.vs + lb * a.sw + lane,
+                        reinterpret_cast<volatile float *>(outv[s & 3])[lane], tg);
             }
         }
-        prefetch(s + 1);
-        // red[s & 1] is next written at task s + 2, after every thread has
-        // passed the barrier of task s + 1
+        if (lane == 0 && head.y) {
+            const size_t e = my_e + (size_t)head.x * NB;
+            if (a.zpair) reinterpret_cast<float2 *>(a.z)[e] = make_float2(acc[0], alo[0]);
+            else a.z[e] = (double)acc[0] + (double)alo[0];
+        }
+        if (++slot == nslot) {
+            slot = 0;
+            par ^= 1u;
+        }
     }
     if (blockIdx.x == 0 && tid == 0) advance_tag(a.tagp, tag0, (unsigned int)a.ntags);
 }
 
-constexpr int SW_CT = 288, SW_CPT = 2, SW_MAXSLOT = 6;
+constexpr int SW_MAXSLOT = 6;
 constexpr size_t SW_SMEM_MAX = 220 * 1024;
 
 // ---------------------------------------------------------------------------
@@ -762,40 +909,92 @@ int sweep_plan(int M, int h, int twisted, SweepPlan &P)
     return BFS_OK;
 }
 
+// The table as the kernel reads it (SweepDev); vs words a slice, nv words of y, which x
+// follows.
+static std::vector<SweepDev> device_table(const SweepPlan &P, int vs, size_t nv)
+{
+    std::vector<SweepDev> out;
+    for (const SweepTask &t : P.tasks) {
+        SweepDev d;
+        memset(&d, 0, sizeof d);
+        int n = 0, order = 0;
+        auto src = [&](int p) { return (t.vec[p] >> 2) & 3; };
+        auto take = [&](int p) {
+            d.blk[n] = make_int4(t.m[p], (int)((t.vec[p] & 1) * nv) + t.m[p] * vs, t.uid[p], 0);
+            order |= ((t.vec[p] >> 1) & 1) << (4 + n);
+            n++;
+        };
+        for (int wi = 0; wi < SW_HW; wi++)
+            for (int p = 0; p < t.nblk; p++)
+                if (src(p) == SW_WIN && ((t.vec[p] >> 4) & 3) == wi) {
+                    take(p);
+                    order |= 1 << wi;
+                }
+        for (int p = 0; p < t.nblk; p++)
+            if (src(p) == SW_EARLY) take(p);
+        for (int p = 0; p < t.nblk; p++)
+            if (src(p) == SW_CRIT) {
+                take(p);
+                order |= 4;
+            }
+        d.head = make_int4(t.k, t.out, t.nblk, order);
+        out.push_back(d);
+    }
+    return out;
+}
+
 using FlowKernel = void (*)(FlowArgs);
 
+// Instances of the task-table kernel by words of a vector slice per poll thread,
+// columns of a lane (4 in every 128) and blocks per task.
+constexpr int SW_PW = 5;
+template <int WPT>
+static FlowKernel pick_sweep_w(int nq, int bm)
+{
+    if (nq == 3) return bm == 4 ? k_apply_sweep<SW_PW, WPT, 3, 4> : k_apply_sweep<SW_PW, WPT, 3, SW_BMAX>;
+    return bm == 4 ? k_apply_sweep<SW_PW, WPT, 5, 4> : k_apply_sweep<SW_PW, WPT, 5, SW_BMAX>;
+}
+static FlowKernel pick_sweep(int wpt, int nq, int bm)
+{
+    return wpt == 2 ? pick_sweep_w<2>(nq, bm) : pick_sweep_w<4>(nq, bm);
+}
+
+template <bool PAIR>
 static FlowKernel pick_flow(int rpc, int cpt)
 {
-    if (rpc <= 4 && cpt <= 2) return k_apply_flow<4, 2>;
-    if (rpc <= 8 && cpt <= 2) return k_apply_flow<8, 2>;
-    if (rpc <= 8 && cpt <= 3) return k_apply_flow<8, 3>;
+    if (rpc <= 4 && cpt <= 2) return k_apply_flow<4, 2, PAIR>;
+    if (rpc <= 8 && cpt <= 2) return k_apply_flow<8, 2, PAIR>;
+    if (rpc <= 8 && cpt <= 3) return k_apply_flow<8, 3, PAIR>;
     return nullptr;
 }
 
 // Shape of the task-table kernel for nb-wide slice blocks, half band h,
 // `groups` CTA groups on G SMs and at most ntask tasks per group (staged in
-// shared memory after the ring); false if its tiles do not take them.
-static bool sweep_shape(int nb, int h, int groups, int G, int ntask, FlowKernel &kern, int &rpc, int &nslot,
-                        size_t &dyn)
+// shared memory after the ring and the vectors); false if its tiles do not take them.
+struct SweepShape {
+    int Gg, rows, sw, wpt, nq, bm, nslot;
+    size_t dyn;
+    int tpb() const { return 32 * (rows + SW_PW + 1); }
+};
+
+static bool sweep_shape(int nb, int h, int groups, int G, int ntask, SweepShape &S)
 {
     const int ldp = (nb + 3) / 4 * 4;
-    if (nb > SW_CT * SW_CPT || h + 1 > SW_BMAX || G < groups) return false;
-    const int Gg = G / groups;  // the smaller group
-    const int rows = (nb + Gg - 1) / Gg;
-    if (rows <= 4) {
-        rpc = 4;
-        kern = k_apply_sweep<SW_CT, 4, SW_CPT>;
-    } else if (rows <= 8) {
-        rpc = 8;
-        kern = k_apply_sweep<SW_CT, 8, SW_CPT>;
-    } else {
-        return false;
-    }
-    const size_t slot = (size_t)SW_BMAX * rpc * ldp * sizeof(float);
-    const size_t tbytes = (size_t)ntask * sizeof(SweepTask);
-    if (tbytes + 2 * slot > SW_SMEM_MAX) return false;
-    nslot = (int)std::min<size_t>(SW_MAXSLOT, (SW_SMEM_MAX - tbytes) / slot);
-    dyn = slot * nslot + tbytes;
+    S.Gg = G / groups;  // CTAs of a group
+    S.bm = h + 1 <= 4 ? 4 : SW_BMAX;
+    S.nq = ldp <= 384 ? 3 : 5;
+    if (nb > 128 * S.nq || h + 1 > S.bm || S.Gg < 1) return false;
+    S.rows = (nb + S.Gg - 1) / S.Gg;
+    if (S.rows > SW_ROWS) return false;
+    S.sw = S.rows <= 4 ? 4 : 8;  // 32- or 64-byte segment of a slice per CTA
+    S.wpt = (S.sw * S.Gg + 32 * SW_PW - 1) / (32 * SW_PW) <= 2 ? 2 : 4;
+    if (S.sw * S.Gg > 32 * SW_PW * S.wpt) return false;
+    const size_t slot = (size_t)(h + 1) * S.rows * ldp * sizeof(float);
+    const size_t rest = (size_t)(2 + 2 * (h + 1)) * ldp * sizeof(float) +
+                        (size_t)ntask * (sizeof(SweepDev) + S.rows * sizeof(float2));
+    if (rest + 2 * slot > SW_SMEM_MAX) return false;
+    S.nslot = (int)std::min<size_t>(SW_MAXSLOT, (SW_SMEM_MAX - rest) / slot);
+    S.dyn = slot * S.nslot + rest;
     return true;
 }
 
@@ -807,16 +1006,13 @@ int sweep_twist_ok(bfs_ctx *c, int h)
     if (h < 1 || c->M - h < 2) return 0;
     SweepPlan P;
     if (sweep_plan(c->M, h, 1, P) != BFS_OK || P.groups != 2) return 0;
-    FlowKernel kern;
-    int rpc, nslot;
-    size_t dyn;
-    if (!sweep_shape(3 * (c->N + 1), h, 2, num_sms(c->device), std::max(P.ntask[0], P.ntask[1]), kern, rpc,
-                     nslot, dyn))
-        return 0;
+    SweepShape S;
+    if (!sweep_shape(c->nb, h, 2, num_sms(c->device), std::max(P.ntask[0], P.ntask[1]), S)) return 0;
+    const FlowKernel kern = pick_sweep(S.wpt, S.nq, S.bm);
     BFS_CUDA_TRY(c, cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)SW_SMEM_MAX));
     int per_sm = 0;
-    BFS_CUDA_TRY(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SW_CT + 32, dyn));
+    BFS_CUDA_TRY(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, S.tpb(), S.dyn));
     return per_sm >= 1 ? 1 : 0;
 }
 
@@ -839,7 +1035,7 @@ __global__ void k_set_tag(unsigned int *p, unsigned int v) { *p = v; }
 int flow_reset(bfs_ctx *c, cudaStream_t s)
 {
     if (!c->d_flow) return BFS_OK;
-    const size_t nv = (size_t)c->M * c->nb;
+    const size_t nv = (size_t)c->M * c->flow_vs;
     BFS_CUDA_TRY(c, cudaMemsetAsync(c->d_flow, 0, sizeof(unsigned long long) * (2 * nv + 1), s));
     k_set_tag<<<1, 1, 0, s>>>(reinterpret_cast<unsigned int *>(c->d_flow + 2 * nv), 1u);
     c->launches++;
@@ -862,7 +1058,6 @@ int precond_make_f32(bfs_ctx *c, cudaStream_t s)
     const int ldp = (c->nb + 3) / 4 * 4;
     const size_t rows = (size_t)c->nb * c->M * (2 * c->pc_h + 1);
     const size_t cnt = rows * ldp;
-    const size_t nv = (size_t)c->M * c->nb;
     c->ldp32 = ldp;
     cudaFree(c->d_pc32);
     cudaFree(c->d_flow);
@@ -871,41 +1066,49 @@ int precond_make_f32(bfs_ctx *c, cudaStream_t s)
     c->d_flow = nullptr;
     c->d_tasks = nullptr;
     c->sweep_table = 0;
+    // the task table: two chains if the factors are in the two-ended order
+    const int twisted = c->pc_twist >= 0;
+    SweepShape S;
+    c->sweep_ntags = 2 * c->M;
+    SweepPlan P;
+    const bool planned = sweep_plan(c->M, c->pc_h, twisted, P) == BFS_OK;  // h < SW_BMAX only
+    if (twisted && (!planned || P.twist != c->pc_twist)) {
+        c->err = "sweep schedule does not match the factor order";
+        return BFS_EINVAL;
+    }
+    const bool table = planned && sweep_shape(c->nb, c->pc_h, twisted ? 2 : 1, num_sms(c->device),
+                                              std::max(P.ntask[0], P.ntask[1]), S);
+    if (twisted && !table) {
+        c->err = "two-ended factors need the task-table sweep kernel";
+        return BFS_EINVAL;
+    }
+    // words of a vector slice: a segment per CTA for the task-table kernel
+    c->flow_vs = table ? S.sw * S.Gg : c->nb;
+    const size_t nv = (size_t)c->M * c->flow_vs;
     if (cudaMalloc(&c->d_pc32, sizeof(float) * cnt) != cudaSuccess ||
         cudaMalloc(&c->d_flow, sizeof(unsigned long long) * (2 * nv + 1)) != cudaSuccess) {
         cudaGetLastError();
         c->err = "FP32 preconditioner copy: out of device memory";
         return BFS_ENOMEM;
     }
-    // the task table: two chains if the factors are in the two-ended order
-    const int twisted = c->pc_twist >= 0;
-    FlowKernel kern;
-    int rpc = 0, nslot = 0;
-    size_t dyn = 0;
-    c->sweep_ntags = 2 * c->M;
-    SweepPlan P;
-    const bool planned = sweep_plan(c->M, c->pc_h, twisted, P) == BFS_OK;  // h <= 3 only
-    if (twisted && (!planned || P.twist != c->pc_twist)) {
-        c->err = "sweep schedule does not match the factor order";
-        return BFS_EINVAL;
-    }
-    if (planned && sweep_shape(c->nb, c->pc_h, twisted ? 2 : 1, num_sms(c->device),
-                               std::max(P.ntask[0], P.ntask[1]), kern, rpc, nslot, dyn)) {
-        BFS_CUDA_TRY(c, cudaMalloc(&c->d_tasks, sizeof(SweepTask) * P.tasks.size()));
-        BFS_CUDA_TRY(c, cudaMemcpy(c->d_tasks, P.tasks.data(), sizeof(SweepTask) * P.tasks.size(),
+    if (table) {
+        c->h_tasks = device_table(P, c->flow_vs, nv);
+        BFS_CUDA_TRY(c, cudaMalloc(&c->d_tasks, sizeof(SweepDev) * c->h_tasks.size()));
+        BFS_CUDA_TRY(c, cudaMemcpy(c->d_tasks, c->h_tasks.data(), sizeof(SweepDev) * c->h_tasks.size(),
                                    cudaMemcpyHostToDevice));
-        c->h_tasks = P.tasks;
         c->sweep_table = 1;
         c->sweep_groups = P.groups;
         c->sweep_ntask[0] = P.ntask[0];
         c->sweep_ntask[1] = P.ntask[1];
         c->sweep_ntags = P.ntask[0] + P.ntask[1];
-        c->sweep_rpc = rpc;
-        c->sweep_nslot = nslot;
-        c->sweep_dyn = dyn;
-    } else if (twisted) {
-        c->err = "two-ended factors need the task-table sweep kernel";
-        return BFS_EINVAL;
+        c->sweep_wpt = S.wpt;
+        c->sweep_nq = S.nq;
+        c->sweep_gg = S.Gg;
+        c->sweep_sw = S.sw;
+        c->sweep_rows = S.rows;
+        c->sweep_bm = S.bm;
+        c->sweep_nslot = S.nslot;
+        c->sweep_dyn = S.dyn;
     }
     int rc = flow_reset(c, s);
     if (rc) return rc;
@@ -930,28 +1133,33 @@ int apply_flow_launch(bfs_ctx *c, const double *r, double *z, cudaStream_t s)
     a.pc = c->d_pc32;
     a.r = r; a.z = z;
     a.Y = c->d_flow;
-    a.X = c->d_flow + (size_t)c->M * c->nb;
-    a.nb = c->nb; a.NB = c->N + 1; a.M = c->M; a.h = c->pc_h;
+    a.X = c->d_flow + (size_t)c->M * c->flow_vs;
+    // condensed blocks: right-hand side and result slice by slice, one field of nb
+    a.nb = c->nb; a.NB = c->pc_cond ? c->nb : c->N + 1; a.M = c->M; a.h = c->pc_h;
     a.ldp = c->ldp32;
-    a.tagp = reinterpret_cast<unsigned int *>(c->d_flow + 2 * (size_t)c->M * c->nb);
+    a.tagp = reinterpret_cast<unsigned int *>(c->d_flow + 2 * (size_t)c->M * c->flow_vs);
     a.flag = c->d_flag;
     a.spin = spin_limit(c);
     a.tasks = c->d_tasks;
     a.ntask0 = c->sweep_ntask[0];
     a.ntask1 = c->sweep_ntask[1];
-    a.G0 = c->sweep_groups == 2 ? G / 2 : G;
+    a.G0 = c->sweep_table ? c->sweep_gg : G;
+    a.sw = c->sweep_sw;
+    a.vs = c->flow_vs;
     a.ntags = c->sweep_ntags;
     a.nslot = c->sweep_nslot;
+    a.rows = c->sweep_rows;
+    a.zpair = c->pc_cond;
     FlowKernel kern;
     int tpb;
     size_t dyn = 0;
     if (c->sweep_table) {
-        kern = c->sweep_rpc == 4 ? k_apply_sweep<SW_CT, 4, SW_CPT> : k_apply_sweep<SW_CT, 8, SW_CPT>;
-        tpb = SW_CT + 32;
+        kern = pick_sweep(c->sweep_wpt, c->sweep_nq, c->sweep_bm);
+        tpb = 32 * (c->sweep_rows + SW_PW + 1);
         dyn = c->sweep_dyn;
     } else {
         const int rpc = (c->nb + G - 1) / G, cpt = (c->nb + FL_TPB - 1) / FL_TPB;
-        kern = pick_flow(rpc, cpt);
+        kern = c->pc_cond ? pick_flow<true>(rpc, cpt) : pick_flow<false>(rpc, cpt);
         tpb = FL_TPB;
         if (!kern) return 0;
     }
@@ -977,18 +1185,20 @@ int apply_flow_launch(bfs_ctx *c, const double *r, double *z, cudaStream_t s)
     // test hook: one wait of this launch is for a vector no task writes
     const bool stall = c->sweep_table && c->dbg_stall_task >= 0 && !c->capturing;
     if (stall) {
-        std::vector<SweepTask> bad = c->h_tasks;
-        SweepTask &t = bad[c->dbg_stall_task];
-        if (t.nblk > 0) t.uid[0] = c->sweep_ntags;  // the tag of the next launch's first task
-        BFS_CUDA_TRY(c, cudaMemcpyAsync(c->d_tasks, bad.data(), sizeof(SweepTask) * bad.size(),
+        std::vector<SweepDev> bad = c->h_tasks;
+        SweepDev &t = bad[c->dbg_stall_task];
+        // the last block's vector: polled for, not one held since an earlier task
+        if (t.head.z > 0) t.blk[t.head.z - 1].z = c->sweep_ntags;  // the tag of the next launch's first task
+        BFS_CUDA_TRY(c, cudaMemcpyAsync(c->d_tasks, bad.data(), sizeof(SweepDev) * bad.size(),
                                         cudaMemcpyHostToDevice, s));
         BFS_CUDA_TRY(c, cudaStreamSynchronize(s));
     }
     void *args[] = {&a};
-    cudaError_t e = cudaLaunchCooperativeKernel((const void *)kern, dim3(G), dim3(tpb), args, dyn, s);
+    const int grid = c->sweep_table ? c->sweep_gg * c->sweep_groups : G;
+    cudaError_t e = cudaLaunchCooperativeKernel((const void *)kern, dim3(grid), dim3(tpb), args, dyn, s);
     if (stall) {
         c->dbg_stall_task = -1;
-        BFS_CUDA_TRY(c, cudaMemcpyAsync(c->d_tasks, c->h_tasks.data(), sizeof(SweepTask) * c->h_tasks.size(),
+        BFS_CUDA_TRY(c, cudaMemcpyAsync(c->d_tasks, c->h_tasks.data(), sizeof(SweepDev) * c->h_tasks.size(),
                                         cudaMemcpyHostToDevice, s));
         BFS_CUDA_TRY(c, cudaStreamSynchronize(s));
     }
@@ -1005,7 +1215,7 @@ extern "C" {
 int bfs_sweep_schedule(int M, int half_band, int twisted, int *tasks_out, int cap, int *ntask_out)
 {
     bfs::SweepPlan P;
-    if (bfs::sweep_plan(M, half_band, twisted, P) != BFS_OK) return BFS_EINVAL;
+    if (half_band > 3 || bfs::sweep_plan(M, half_band, twisted, P) != BFS_OK) return BFS_EINVAL;
     if (ntask_out) {
         ntask_out[0] = P.ntask[0];
         ntask_out[1] = P.ntask[1];
@@ -1013,8 +1223,15 @@ int bfs_sweep_schedule(int M, int half_band, int twisted, int *tasks_out, int ca
     const int n = (int)P.tasks.size();
     if (tasks_out) {
         if (cap < n) return BFS_EINVAL;
-        static_assert(sizeof(bfs::SweepTask) == sizeof(int) * (4 + 3 * bfs::SW_BMAX), "task layout");
-        memcpy(tasks_out, P.tasks.data(), sizeof(bfs::SweepTask) * n);
+        for (int i = 0; i < n; i++) {  // 16 ints a task: at most 4 blocks for half_band <= 3
+            const bfs::SweepTask &t = P.tasks[i];
+            int *o = tasks_out + 16 * i;
+            const int head[4] = {t.k, t.out, t.nblk, 0};
+            memcpy(o, head, sizeof head);
+            memcpy(o + 4, t.m, 4 * sizeof(int));
+            memcpy(o + 8, t.vec, 4 * sizeof(int));
+            memcpy(o + 12, t.uid, 4 * sizeof(int));
+        }
     }
     return n;
 }
@@ -1026,7 +1243,7 @@ int bfs_debug_stall_sweep(bfs_ctx *c, int task)
         c->err = "the stall hook needs the FP32 task-table sweeps";
         return BFS_EINVAL;
     }
-    if (task < 0 || task >= (int)c->h_tasks.size() || c->h_tasks[task].nblk == 0) {
+    if (task < 0 || task >= (int)c->h_tasks.size() || c->h_tasks[task].head.z == 0) {
         c->err = "no waiting block in that task";
         return BFS_EINVAL;
     }

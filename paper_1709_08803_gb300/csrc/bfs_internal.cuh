@@ -66,12 +66,21 @@ struct BatchVariant {
 //          bits 2-3: where a thread finds its columns of v_p (SW_EARLY, SW_WIN,
 //          SW_CRIT); bits 4-5: the register-window index (SW_WIN)
 //   uid[p]: the task that wrote v_p (tasks are numbered group 0 first)
-constexpr int SW_BMAX = 4;
+constexpr int SW_BMAX = 7;  // blocks per task: half bands up to 6
 constexpr int SW_HW = 2;  // register window: the last SW_HW critical vectors
 enum { SW_EARLY = 0, SW_WIN = 1, SW_CRIT = 2 };
 struct SweepTask {
-    int k, out, nblk, pad;
+    int k, out, nblk;
     int m[SW_BMAX], vec[SW_BMAX], uid[SW_BMAX];
+};
+
+// A task as the kernel reads it, in 16-byte words: head {k, out, nblk, order} and
+// per block {m, word offset of its vector from y, uid, 0}, blocks in the order
+// SW_WIN (newest first), SW_EARLY, SW_CRIT.  order: bits 0-1 the register-window
+// entries used, bit 2 a critical block, bit 4 + p the sign of block p (1: plus).
+struct SweepDev {
+    int4 head;
+    int4 blk[SW_BMAX];
 };
 
 struct SweepPlan {
@@ -142,10 +151,12 @@ struct bfs_ctx {
     unsigned long long flow_count;  // FP32 sweep launches since the tags were reset
     int capturing;               // a CUDA graph is being captured on the solver stream
     int pc_twist;                // two-ended factor order: first middle slice; -1: one-ended
-    bfs::SweepTask *d_tasks;     // task table of the FP32 sweeps
-    std::vector<bfs::SweepTask> h_tasks;
+    bfs::SweepDev *d_tasks;      // task table of the FP32 sweeps
+    std::vector<bfs::SweepDev> h_tasks;
     int sweep_table;             // 1: the task-table kernel runs the FP32 sweeps
-    int sweep_groups, sweep_ntask[2], sweep_ntags, sweep_rpc, sweep_nslot;
+    int sweep_groups, sweep_ntask[2], sweep_ntags, sweep_nslot;
+    int sweep_gg, sweep_sw, sweep_wpt, sweep_nq, sweep_rows, sweep_bm;  // shape of the task-table kernel
+    int flow_vs;                 // words of a slice of the tagged vectors
     size_t sweep_dyn;
     int dbg_stall_task;          // test hook: task whose first wait is made unsatisfiable, or -1
 
@@ -173,6 +184,11 @@ struct bfs_ctx {
     void *d_gjscr;     // dataflow Gauss-Jordan: candidate slots, perm / pinv
     double *d_gjdata;  // dataflow Gauss-Jordan: candidate rows
     double *d_rowsum5; // Nt
+    // condensed slice blocks (condense.cu): phi_x eliminated, nb = 2 (N+1) + 1
+    int pc_cond;
+    double pc_F;       // Froude number the preconditioner was factored for
+    double *d_ktab;    // tables of K5, K7, K6, then scratch and K6 in float pairs
+    double *d_rc, *d_zc;  // reduced right-hand side and solution, M nb each
     int *d_pivflag;
     double *d_perm_a, *d_perm_b;  // n each
 
@@ -212,6 +228,14 @@ extern const int kNumBatchVariants;
 int batch_pairs_occupancy(int v, int *blocks_per_sm);
 void batch_pairs_launch(int v, int grid, const BatchInst *inst, const int4 *items, int n_items,
                         unsigned int *counter, const unsigned char *mask, cudaStream_t s);
+
+// condense.cu
+int cond_ok(const bfs_ctx *c);
+int cond_fits(const bfs_ctx *c, int h);
+int cond_tables(bfs_ctx *c, cudaStream_t s);
+int cond_form(bfs_ctx *c, cudaStream_t s);
+int cond_pre(bfs_ctx *c, const double *r, cudaStream_t s);
+int cond_post(bfs_ctx *c, const double *r, double *z, cudaStream_t s);
 
 // pairs_df64.cu
 PairPlan plan_df(int Nt, int Ns, int splits_req, int sms);

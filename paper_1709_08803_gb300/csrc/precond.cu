@@ -83,8 +83,8 @@ __device__ double rect_S2_pc(double s1, double s2, double t1, double t2)
     return g_K5(s2, t2) - g_K5(s1, t2) - g_K5(s2, t1) + g_K5(s1, t1);
 }
 
-// Row sums of w K5 over all nodes (and images) minus the closed-form integral:
-// the coefficient of zeta_x* in the linear F2.
+// Row sums of w K5 over all nodes and images (in out: cond_tables) minus the
+// closed-form integral: the coefficient of zeta_x* in the linear F2.
 __global__ void k_rowsum5(PcArgs a, double *out)
 {
     int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -92,16 +92,7 @@ __global__ void k_rowsum5(PcArgs a, double *out)
     if (e >= Nt) return;
     int k = e % (a.N - 1), l = e / (a.N - 1);
     double xs = a.x1 + (k + 0.5) * a.dx, ys = a.y1 + l * a.dy;
-    double acc = 0.0;
-    for (int img = 0; img < (a.half ? 2 : 1); img++)
-        for (int j = (img ? 1 : 0); j < a.M; j++) {
-            double t = (img ? -1.0 : 1.0) * (a.y1 + j * a.dy) - ys;
-            for (int i = 0; i < a.N; i++) {
-                double s = a.x1 + i * a.dx - xs;
-                acc += trap_w(a, i, j) * rsqrt(s * s + t * t);
-            }
-        }
-    out[e] = acc - rect_S2_pc(a.x1 - xs, a.xhi - xs, a.ylo - ys, a.yhi - ys);
+    out[e] -= rect_S2_pc(a.x1 - xs, a.xhi - xs, a.ylo - ys, a.yhi - ys);
 }
 
 // Dense entries of block (l, m): one CTA per (l, d, k), threads over source nodes n.
@@ -1392,7 +1383,7 @@ __global__ void __launch_bounds__(AP_TPB, 1) k_apply_coop(ApplyArgs a)
     __shared__ double red[AP_WARPS];
     const int nb = a.nb, NB = a.NB, M = a.M, h = a.h, nd = 2 * h + 1;
     const size_t bsz = (size_t)nb * nb;
-    const int n = 3 * NB * M;
+    const int n = nb * M;
     const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gstride = gridDim.x * blockDim.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rpc = (nb + gridDim.x - 1) / gridDim.x;                   // rows per CTA
@@ -1493,7 +1484,7 @@ __global__ void __launch_bounds__(AP_TPB, 1) k_apply_coop(ApplyArgs a)
 static PcArgs pc_args(const bfs_ctx *c, int h)
 {
     PcArgs a;
-    a.N = c->N; a.M = c->M; a.half = c->half; a.h = h; a.nb = 3 * (c->N + 1);
+    a.N = c->N; a.M = c->M; a.half = c->half; a.h = h; a.nb = c->nb;
     a.x1 = c->x1; a.y1 = c->y1; a.dx = c->dx; a.dy = c->dy; a.F = c->F; a.n_rad = c->opt.n_rad;
     a.xhi = c->x1 + (c->N - 1) * c->dx;
     a.yhi = c->y1 + (c->M - 1) * c->dy;
@@ -1522,6 +1513,9 @@ void precond_free(bfs_ctx *c)
     c->d_gjscr = nullptr;
     c->d_gjdata = nullptr;
     cudaFree(c->d_rowsum5);
+    cudaFree(c->d_ktab);
+    cudaFree(c->d_rc);
+    c->d_ktab = c->d_rc = c->d_zc = nullptr;
     cudaFree(c->d_pivflag);
     cudaFree(c->d_perm_a);
     c->d_pc = c->d_gj = c->d_rowsum5 = c->d_perm_a = c->d_perm_b = nullptr;
@@ -1691,7 +1685,11 @@ int precond_factor(bfs_ctx *c, int half_band, cudaStream_t s)
     if (h > c->M - 1) h = c->M - 1;
     if (h > 16) h = 16;  // the sweep kernel takes at most 17 blocks per row
     precond_free(c);
-    const int nb = 3 * (c->N + 1), M = c->M, nd = 2 * h + 1;
+    // phi_x taken out of the slice blocks wherever that is an exact elimination
+    // with a sound pivot (condense.cu)
+    c->pc_cond = cond_ok(c) && cond_fits(c, h);
+    c->pc_F = c->F;
+    const int nb = c->pc_cond ? 2 * (c->N + 1) + 1 : 3 * (c->N + 1), M = c->M, nd = 2 * h + 1;
     c->nb = nb;
     c->pc_h = h;
     // the two-ended order whenever the FP32 task-table sweeps can run its two chains
@@ -1724,13 +1722,17 @@ int precond_factor(bfs_ctx *c, int half_band, cudaStream_t s)
     BFS_CUDA_TRY(c, cudaMemsetAsync(c->d_pivflag, 0, sizeof(int) * 8, s));
 
     PcArgs a = pc_args(c, h);
-    k_rowsum5<<<(c->Nt + 127) / 128, 128, 0, s>>>(a, c->d_rowsum5);
+    if ((rc = cond_tables(c, s))) return rc;
+    k_rowsum5<<<(c->Nt + 63) / 64, 64, 0, s>>>(a, c->d_rowsum5);
     c->launches++;
-    k_form_dense<<<dim3(c->N - 1, nd, M), 128, sizeof(double) * (2 * c->N + 1), s>>>(a, c->d_pc,
-                                                                                  c->d_rowsum5);
-    c->launches++;
-    k_form_sparse<<<(M * nb + 127) / 128, 128, 0, s>>>(a, c->d_pc);
-    c->launches++;
+    if (c->pc_cond) {
+        if ((rc = cond_form(c, s))) return rc;
+    } else {
+        k_form_dense<<<dim3(c->N - 1, nd, M), 128, sizeof(double) * (2 * c->N + 1), s>>>(a, c->d_pc,
+                                                                                      c->d_rowsum5);
+        k_form_sparse<<<(M * nb + 127) / 128, 128, 0, s>>>(a, c->d_pc);
+        c->launches += 2;
+    }
     if (a.tau != 0.0) {
         k_form_tension<<<(M * (c->N - 1) + 127) / 128, 128, 0, s>>>(a, c->d_pc);
         c->launches++;
@@ -1920,11 +1922,20 @@ int precond_apply(bfs_ctx *c, const double *r, double *z, cudaStream_t s)
         c->ev_kind.push_back(3);
         cudaEventRecord(ev0, s);
     }
-    const int split = apply_flow_launch(c, r, z, s);
+    const double *rhs = r;
+    double *sol = z;
+    int rc = BFS_OK;
+    if (c->pc_cond) {
+        if ((rc = cond_pre(c, r, s))) return rc;
+        rhs = c->d_rc;
+        sol = c->d_zc;
+    }
+    const int split = apply_flow_launch(c, rhs, sol, s);
     if (split < 0) return split;
     if (split == 1) {
+        if (c->pc_cond) rc = cond_post(c, r, z, s);
         if (ev1) cudaEventRecord(ev1, s);
-        return BFS_OK;
+        return rc;
     }
     if (c->pc_twist >= 0) {
         c->err = "two-ended factors need the FP32 sweep kernel";
@@ -1940,8 +1951,8 @@ int precond_apply(bfs_ctx *c, const double *r, double *z, cudaStream_t s)
         c->apply_grid = num_sms(c->device);  // one 1024-thread CTA per SM
     }
     ApplyArgs a;
-    a.pc = c->d_pc; a.r = r; a.z = z; a.x = c->d_perm_a; a.y = c->d_perm_b;
-    a.nb = c->nb; a.NB = c->N + 1; a.M = c->M; a.h = c->pc_h;
+    a.pc = c->d_pc; a.r = rhs; a.z = sol; a.x = c->d_perm_a; a.y = c->d_perm_b;
+    a.nb = c->nb; a.NB = c->pc_cond ? c->nb : c->N + 1; a.M = c->M; a.h = c->pc_h;
     a.bar = reinterpret_cast<CoopBar *>(c->d_pivflag + 4);
     a.flag = c->d_flag;
     a.spin = wait_spin(c);
@@ -1950,8 +1961,9 @@ int precond_apply(bfs_ctx *c, const double *r, double *z, cudaStream_t s)
     BFS_CUDA_TRY(c, cudaLaunchCooperativeKernel((const void *)k_apply_coop, dim3(c->apply_grid),
                                                 dim3(AP_TPB), args, 0, s));
     c->launches++;
+    if (c->pc_cond) rc = cond_post(c, r, z, s);
     if (ev1) cudaEventRecord(ev1, s);
-    return BFS_OK;
+    return rc;
 }
 
 }  // namespace bfs
