@@ -41,6 +41,7 @@ void free_all(bfs_ctx *c)
     cudaFree(c->d_red);
     cudaFree(c->d_tailbar);
     cudaFree(c->d_V);
+    cudaFree(c->d_Z);
     cudaFree(c->d_H);
     cudaFree(c->d_giv);
     cudaFree(c->d_sbase);

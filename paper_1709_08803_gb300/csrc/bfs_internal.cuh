@@ -134,6 +134,7 @@ struct bfs_ctx {
     // Newton / GMRES workspace
     int m_alloc;
     double *d_V;      // (m+1) n Krylov basis
+    double *d_Z;      // m n preconditioned basis vectors z_j = P^-1 v_j
     double *d_H;      // Hessenberg, column j at d_H + j (m+1)
     double *d_giv;    // cs[m], sn[m], g[m+1], y[m], h[m+1], h2[m+1]
     double *d_red;    // reduction partials

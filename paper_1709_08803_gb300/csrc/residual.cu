@@ -339,8 +339,8 @@ __device__ __forceinline__ void pair_tile(const double *__restrict__ src, int pe
 
 // ---------------------------------------------------------------------------
 // FP32C all-pairs with the packed FP32x2 arithmetic of sm_100-class GPUs: one
-// instruction applies the same operation to two sources, so the 42 FP32
-// operations of an index pair take 21 issue slots (the five reciprocal square
+// instruction applies the same operation to two sources, so the 45 FP32
+// operations of an index pair take 23 issue slots (the five reciprocal square
 // roots stay scalar on the special-function unit); the FMA pipe still spends
 // one lane-cycle per operation, and it is the kernel's limit.  The quadratic
 // form of S2 is taken as s^2 + t^2 + (zeta_x* s + zeta_y* t)^2 (three
@@ -418,6 +418,8 @@ __device__ __forceinline__ void pair_tile_x2(const float *__restrict__ src, int 
                                              int *flag)
 {
     static_assert(CH % 2 == 0, "sources are taken in pairs");
+    constexpr int NSUM = 5;  // sums of a chunk: double and single layers apart (joined in FP32
+                             // they lose a tenth of the bottom rows' accuracy), S2
     constexpr unsigned int CHUNK_BYTES = CH * REC * sizeof(float);
     const float *sb = src + (size_t)split * per_split * REC;
     const int nch = per_split / CH;
@@ -457,11 +459,11 @@ __device__ __forceinline__ void pair_tile_x2(const float *__restrict__ src, int 
             return;
         }
         const f2 *sp2 = reinterpret_cast<const f2 *>(ring.at(q));
-        f2 L[TPT][NACC];
+        f2 L[TPT][NSUM];
 #pragma unroll
         for (int p = 0; p < TPT; p++)
 #pragma unroll
-            for (int qq = 0; qq < NACC; qq++) L[p][qq].v = 0ull;
+            for (int qq = 0; qq < NSUM; qq++) L[p][qq].v = 0ull;
 #pragma unroll 2
         for (int i = 0; i < CH / 2; i++) {
             const f2 *r = sp2 + i * REC;
@@ -477,44 +479,52 @@ __device__ __forceinline__ void pair_tile_x2(const float *__restrict__ src, int 
                 {
                     const f2 d = f2_sub(zs, TZ[p]);
                     const f2 ri = f2_rsq(f2_fma(d, d, rho2));
+                    const f2 ri3 = f2_mul(f2_mul(ri, ri), ri);
                     const f2 num = f2_fma(sy, zys, f2_fma(sx, zxs, d));
-                    const f2 t = f2_mul(f2_fma(NTF[p], w1, w1f), num);
-                    L[p][0] = f2_fma(f2_fma(t, f2_mul(ri, ri), w2zx), ri, L[p][0]);
+                    const f2 dens = f2_fma(NTF[p], w1, w1f);
+                    L[p][0] = f2_fma(f2_mul(dens, num), ri3, L[p][0]);
+                    L[p][1] = f2_fma(w2zx, ri, L[p][1]);
                     // A s^2 + B s t + C t^2 = s^2 + t^2 + (zeta_x* s + zeta_y* t)^2
                     const f2 mq = f2_fma(ZX[p], sx, f2_mul(ZY[p], sy));
-                    L[p][1] = f2_fma(w2, f2_rsq(f2_fma(mq, mq, rho2)), L[p][1]);
+                    L[p][2] = f2_fma(w2, f2_rsq(f2_fma(mq, mq, rho2)), L[p][2]);
                 }
                 // top target, bottom source: -w g K1(beta) + w sigma beta_x K2(beta)
                 {
                     const f2 d = f2_sub(bs, CTB[p]);
                     const f2 ri = f2_rsq(f2_fma(d, d, rho2));
+                    const f2 ri3 = f2_mul(f2_mul(ri, ri), ri);
                     const f2 num = f2_fma(sy, bys, f2_fma(sx, bxs, d));
-                    L[p][0] = f2_fma(f2_fma(f2_mul(nw1g, num), f2_mul(ri, ri), w2sb), ri, L[p][0]);
+                    L[p][0] = f2_fma(f2_mul(nw1g, num), ri3, L[p][0]);
+                    L[p][1] = f2_fma(w2sb, ri, L[p][1]);
                 }
                 // bottom target, top source: w f K1 + w zeta_x K2
                 {
                     const f2 d = f2_sub(zs, CBT[p]);
                     const f2 ri = f2_rsq(f2_fma(d, d, rho2));
+                    const f2 ri3 = f2_mul(f2_mul(ri, ri), ri);
                     const f2 num = f2_fma(sy, zys, f2_fma(sx, zxs, d));
-                    L[p][2] = f2_fma(f2_fma(f2_mul(w1f, num), f2_mul(ri, ri), w2zx), ri, L[p][2]);
+                    L[p][3] = f2_fma(f2_mul(w1f, num), ri3, L[p][3]);
+                    L[p][4] = f2_fma(w2zx, ri, L[p][4]);
                 }
                 // bottom target, bottom source: -w (g - g*) K1(beta)
                 {
                     const f2 d = f2_sub(bs, TB[p]);
                     const f2 ri = f2_rsq(f2_fma(d, d, rho2));
+                    const f2 ri3 = f2_mul(f2_mul(ri, ri), ri);
                     const f2 num = f2_fma(sy, bys, f2_fma(sx, bxs, d));
                     const f2 densn = f2_fma(TG[p], w1, nw1g);  // g* w - w g
-                    L[p][2] = f2_fma(f2_mul(f2_mul(densn, num), f2_mul(ri, ri)), ri, L[p][2]);
+                    L[p][3] = f2_fma(f2_mul(densn, num), ri3, L[p][3]);
                 }
             }
         }
 #pragma unroll
         for (int p = 0; p < TPT; p++)
 #pragma unroll
-            for (int qq = 0; qq < NACC; qq++) {
+            for (int qq = 0; qq < NSUM; qq++) {
                 float a, b;
                 f2_unpack(L[p][qq], a, b);
-                two_sum_acc(hi[p][qq], lo[p][qq], a + b);
+                // double and single layer of a sheet end in one accumulator
+                two_sum_acc(hi[p][qq < 2 ? 0 : qq == 2 ? 1 : 2], lo[p][qq < 2 ? 0 : qq == 2 ? 1 : 2], a + b);
             }
         __syncthreads();  // every thread is done with this buffer before it is refilled
     }

@@ -209,15 +209,15 @@ __global__ void k_gemv_sub(double *__restrict__ w, const double *__restrict__ V,
     }
 }
 
-// x = V[0..cnt) y
-__global__ void k_gemv(double *__restrict__ x, const double *__restrict__ V, size_t ldv,
-                       const double *__restrict__ y, int cnt, int n)
+// x += V[0..cnt) y
+__global__ void k_gemv_add(double *__restrict__ x, const double *__restrict__ V, size_t ldv,
+                           const double *__restrict__ y, int cnt, int n)
 {
     __shared__ double ys[128];
     for (int j = threadIdx.x; j < cnt; j += blockDim.x) ys[j] = y[j];
     __syncthreads();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double acc = 0.0;
+        double acc = x[i];
         for (int j = 0; j < cnt; j++) acc = fma(ys[j], V[(size_t)j * ldv + i], acc);
         x[i] = acc;
     }
@@ -438,6 +438,7 @@ int alloc_solver(bfs_ctx *c)
     const int m = c->opt.gmres_restart, n = c->n;
     c->m_alloc = m;
     BFS_CUDA_TRY(c, cudaMalloc(&c->d_V, sizeof(double) * (size_t)(m + 1) * n));
+    BFS_CUDA_TRY(c, cudaMalloc(&c->d_Z, sizeof(double) * (size_t)m * n));
     BFS_CUDA_TRY(c, cudaMalloc(&c->d_H, sizeof(double) * (size_t)(m + 1) * m));
     BFS_CUDA_TRY(c, cudaMalloc(&c->d_giv, sizeof(double) * (size_t)(6 * m + 4)));
     BFS_CUDA_TRY(c, cudaMalloc(&c->d_sbase, sizeof(double) * (size_t)8 * n));
@@ -561,10 +562,16 @@ void gm_cycle_begin(bfs_ctx *c, Gm &g, double beta, cudaStream_t s)
     g.state = Gm::ARNOLDI;
 }
 
+// z_j = P^-1 v_j, kept for the end of the cycle (flexible GMRES, Saad, SIAM J. Sci.
+// Comput. 14, 1993): the update is sum y_j z_j of the very z_j that J multiplied, so
+// the rounding of the FP32 sweeps does not enter it, and a cycle ends without
+// another apply.
+static double *gm_z(bfs_ctx *c, const Gm &g) { return c->d_Z + (size_t)g.j * c->n; }
+
 // Arnoldi step, before the residual: z = P^-1 v_j, then u + h z into d_up.
 int gm_arnoldi_sweep(bfs_ctx *c, Gm &g, cudaStream_t s)
 {
-    int rc = precond_apply(c, c->d_V + (size_t)g.j * c->n, c->d_z, s);
+    int rc = precond_apply(c, c->d_V + (size_t)g.j * c->n, gm_z(c, g), s);
     if (rc) return rc;
     g.precs++;
     return BFS_OK;
@@ -574,7 +581,7 @@ int gm_arnoldi_pre(bfs_ctx *c, Gm &g, cudaStream_t s)
 {
     int rc = gm_arnoldi_sweep(c, g, s);
     if (rc) return rc;
-    return jv_prep(c, g.u, c->d_z, 0.0, c->opt.krylov_precision, s, true);
+    return jv_prep(c, g.u, gm_z(c, g), 0.0, c->opt.krylov_precision, s, true);
 }
 
 // Arnoldi step, after F(u + h z) is in d_Fp: w = J z, CGS2, V_{j+1}, Givens.
@@ -684,7 +691,7 @@ int gm_multi_pre(bfs_ctx *const *cs, Gm *const *gs, int cnt, cudaStream_t s)
             bfs_ctx *c = cs[o + q];
             double h_rel = c->opt.jv_h_rel;
             if (!(h_rel > 0.0)) h_rel = c->opt.krylov_precision == BFS_FP32C ? 3.4526698e-4 : 1.4901161193847656e-8;
-            set.in[q] = MjvInst{gs[o + q]->u, c->d_z, c->d_up, c->d_red, c->d_scal, c->n, h_rel};
+            set.in[q] = MjvInst{gs[o + q]->u, gm_z(c, *gs[o + q]), c->d_up, c->d_red, c->d_scal, c->n, h_rel};
             nmax = std::max(nmax, c->n);
         }
         k_mjv_norms<<<dim3(RED_BLOCKS, set.cnt), RED_TPB, 0, s>>>(set);
@@ -760,19 +767,14 @@ void gm_arnoldi_host(bfs_ctx *c, Gm &g, double hn, double res)
     if (res <= g.target || hn == 0.0 || g.j >= c->m_alloc || g.its >= g.maxit) g.state = Gm::CYCLE_END;
 }
 
-// End of a cycle: du += P^-1 V y.  Then either done, or a restart needs
+// End of a cycle: du += Z y.  Then either done, or a restart needs
 // J du (prepared here: u + h du into d_up; the caller evaluates its residual).
 int gm_cycle_end(bfs_ctx *c, Gm &g, cudaStream_t s)
 {
     const int m = c->m_alloc, n = c->n;
     k_trisolve<<<1, 1, 0, s>>>(c->d_H, c->d_giv, m, g.j);
     c->launches++;
-    k_gemv<<<grid_for(n), 256, 0, s>>>(c->d_w, c->d_V, (size_t)n, c->d_giv + 3 * m + 1, g.j, n);
-    c->launches++;
-    int rc = precond_apply(c, c->d_w, c->d_z, s);
-    if (rc) return rc;
-    g.precs++;
-    k_axpby<<<grid_for(n), 256, 0, s>>>(c->d_du, c->d_du, c->d_z, n, 1.0, 1.0, nullptr);
+    k_gemv_add<<<grid_for(n), 256, 0, s>>>(c->d_du, c->d_Z, (size_t)n, c->d_giv + 3 * m + 1, g.j, n);
     c->launches++;
     if (g.res <= g.target || g.its >= g.maxit) {
         g.state = Gm::DONE;
