@@ -129,7 +129,10 @@ typedef struct {
                               default of Sec. 5's solver), eta_k = | |F_k| - |F_{k-1} +
                               J s_{k-1}| | / |F_{k-1}|, safeguarded by eta_{k-1}^1.618
                               when that exceeds 0.1, kept in [eta, 0.9]; eta_0 =
-                              max(eta, 0.1) */
+                              max(eta, 0.1).  Where eta_k |F_k|_inf <= 5 tol the step
+                              goes on to 0.1 tol, and with a Krylov precision below the
+                              outer one an iterate between 0.2 tol and tol gets one
+                              more step of at most 12 Krylov iterations */
     int wait_polls;        /* polls of a device-side wait (the tags of the preconditioner
                               sweeps, the grid barriers of the cooperative kernels) before
                               it gives up: the kernel raises the context's timeout bit,

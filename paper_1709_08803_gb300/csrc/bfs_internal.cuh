@@ -141,7 +141,7 @@ struct bfs_ctx {
     unsigned int *d_tailbar;  // grid barrier of the fused Arnoldi tail
     int tail_grid;            // its grid (0: the kernels one by one)
     double *d_sbase;  // one allocation holding the n-vectors below
-    double *d_F, *d_du, *d_ut, *d_Ft, *d_z, *d_w, *d_F32, *d_uio;  // n each
+    double *d_F, *d_du, *d_ut, *d_Ft, *d_w, *d_F32, *d_uio;  // n each
     double *h_pin;    // pinned host scalars
 
     // preconditioner
@@ -251,6 +251,7 @@ struct Gm {
     int maxit, its, j, status, precs, jvs;
     State state;
 };
+double gm_last_eta(const bfs_options &o, double finf, double eta);
 void gm_start(bfs_ctx *c, Gm &g, const double *u, const double *F, const double *Fbase,
               double fnorm2, double eta, int maxit, cudaStream_t s);
 void gm_cycle_begin(bfs_ctx *c, Gm &g, double beta, cudaStream_t s);

@@ -521,9 +521,6 @@ static size_t conv_smem(const bfs_ctx *c, int h, size_t k, size_t g) { return (s
 // blocks: 1.2e-7 / 1.3e-7 at 181, 1.4e-7 / 1.4e-7 at 241, 2.9e-7 / 1.3e-7 at 361).
 int cond_fits(const bfs_ctx *c, int h)
 {
-#ifdef NOCOND
-    return 0;
-#endif
     if (c->opt.precond_precision == BFS_FP32C ? (c->N < 140 || c->N > 256) : c->N < 100) return 0;
     return conv_smem(c, h, 8, 8) <= 200 * 1024 && sizeof(double) * (4 * (size_t)c->N + 8) <= 200 * 1024;
 }
