@@ -22,32 +22,41 @@ namespace bfs {
 // Unpack: per slice j and field q, q(x1) followed by q_x at the N nodes; the
 // nodal values follow by the trapezoid rule along x (Sec. 3.1).
 // ---------------------------------------------------------------------------
-__global__ void k_unpack(const double *__restrict__ u, double *__restrict__ nodal, int N, int M,
-                         double dx)
+// One CTA per (field, slice).  The inclusive scan costs FP64 additions (two per
+// clock and SM) and their latency, so it is one pass of shuffles per 256 nodes
+// and a short sum over the warps' totals, instead of a chain of passes in one warp.
+constexpr int UNP_TPB = 256;
+__global__ void __launch_bounds__(UNP_TPB) k_unpack(const double *__restrict__ u, double *__restrict__ nodal, int N,
+                                                    int M, double dx)
 {
-    // one warp per (field, slice): inclusive shuffle scan of the trapezoid increments
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= 3 * M) return;
-    const int f = warp / M, j = warp - f * M;
+    __shared__ double tot[UNP_TPB / 32];
+    const int f = blockIdx.x / M, j = blockIdx.x - f * M, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t NM = (size_t)N * M;
     const double *s = u + (size_t)f * (N + 1) * M + (size_t)j * (N + 1);
     double *q = nodal + (size_t)(3 * f) * NM + (size_t)j * N;
     double *qx = nodal + (size_t)(3 * f + 1) * NM + (size_t)j * N;
     double carry = s[0];
-    for (int i0 = 0; i0 < N; i0 += 32) {
-        const int i = i0 + lane;
+    for (int i0 = 0; i0 < N; i0 += UNP_TPB) {
+        const int i = i0 + threadIdx.x;
         const double cur = i < N ? s[1 + i] : 0.0;
         double inc = (i >= 1 && i < N) ? 0.5 * dx * (s[i] + cur) : 0.0;
+#pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const double v = __shfl_up_sync(0xffffffffu, inc, o);
             if (lane >= o) inc += v;
         }
-        const double val = carry + inc;
+        if (lane == 31) tot[warp] = inc;
+        __syncthreads();
+        double before = carry;
+        for (int w = 0; w < warp; w++) before += tot[w];
         if (i < N) {
-            q[i] = val;
+            q[i] = before + inc;
             qx[i] = cur;
         }
-        carry = __shfl_sync(0xffffffffu, val, 31);
+        if (i0 + UNP_TPB < N) {
+            for (int w = 0; w < UNP_TPB / 32; w++) carry += tot[w];
+            __syncthreads();
+        }
     }
 }
 
@@ -569,45 +578,29 @@ k_pairs64(const double *__restrict__ src, int per_split, const double *__restric
 // (2As + Bt + 2 sqrt(AQ)) (2 sqrt(AQ) - 2As - Bt) = (4AC - B^2) t^2 as
 // ln((4AC - B^2) t^2 / (2 sqrt(AQ) - 2As - Bt)), and t ln(.) -> 0 at t = 0.
 // ---------------------------------------------------------------------------
-__device__ double antideriv_S2(double A, double B, double C, double s, double t)
-{
-    const double Q = A * s * s + B * s * t + C * t * t;
-    const double D = 4.0 * A * C - B * B;
-    double g = 0.0;
-    if (t != 0.0) {
-        const double lin = 2.0 * A * s + B * t, r = 2.0 * sqrt(A * Q);
-        // lin + r = D t^2 / (r - lin): one logarithm, no cancellation when lin < 0
-        const double L = log((lin >= 0.0) ? lin + r : D * t * t / (r - lin));
-        g += t * rsqrt(A) * L;
-    }
-    if (s != 0.0) {
-        const double lin = 2.0 * C * t + B * s, r = 2.0 * sqrt(C * Q);
-        const double L = log((lin >= 0.0) ? lin + r : D * s * s / (r - lin));
-        g += s * rsqrt(C) * L;
-    }
-    return g;
-}
+// sqrt by the reciprocal root above (0 at 0)
+__device__ __forceinline__ double sqrt64(double a) { return a == 0.0 ? 0.0 : a * rsq64(a); }
 
-// One of the two logarithmic terms of antideriv_S2 at corner (s, t): which = 0
-// the t term, 1 the s term (their sum is antideriv_S2).
-__device__ double antideriv_S2_term(double A, double B, double C, double s, double t, int which)
+// One edge of the rectangle in rect_S2: t / sqrt(a) times the logarithm of the
+// ratio of the antiderivative's arguments 2 a s + B t + 2 sqrt(a Q) at s2 and s1,
+// Q = a s^2 + B s t + c t^2 (0 at t = 0).  An argument that would cancel enters as
+// (4 a c - B^2) t^2 / (2 sqrt(a Q) - 2 a s - B t), so the ratio is one quotient of
+// products without cancellation and the edge costs one logarithm, not two.
+__device__ double edge_S2(double a, double B, double c, double s1, double s2, double t)
 {
-    const double Q = A * s * s + B * s * t + C * t * t;
-    const double D = 4.0 * A * C - B * B;
-    if (which == 0) {
-        if (t == 0.0) return 0.0;
-        const double lin = 2.0 * A * s + B * t, r = 2.0 * sqrt(A * Q);
-        return t * rsqrt(A) * log((lin >= 0.0) ? lin + r : D * t * t / (r - lin));
-    }
-    if (s == 0.0) return 0.0;
-    const double lin = 2.0 * C * t + B * s, r = 2.0 * sqrt(C * Q);
-    return s * rsqrt(C) * log((lin >= 0.0) ? lin + r : D * s * s / (r - lin));
+    if (t == 0.0) return 0.0;
+    const double Bt = B * t, ct2 = c * t * t, D = (4.0 * a * c - B * B) * (t * t);
+    const double l2 = fma(2.0 * a, s2, Bt), r2 = 2.0 * sqrt64(a * fma(s2, fma(a, s2, Bt), ct2));
+    const double l1 = fma(2.0 * a, s1, Bt), r1 = 2.0 * sqrt64(a * fma(s1, fma(a, s1, Bt), ct2));
+    const double num = (l2 >= 0.0 ? l2 + r2 : D) * (l1 >= 0.0 ? 1.0 : r1 - l1);
+    const double den = (l2 >= 0.0 ? 1.0 : r2 - l2) * (l1 >= 0.0 ? l1 + r1 : D);
+    return t * rsq64(a) * log(num / den);
 }
 
 __device__ double rect_S2(double A, double B, double C, double s1, double s2, double t1, double t2)
 {
-    return antideriv_S2(A, B, C, s2, t2) - antideriv_S2(A, B, C, s1, t2) -
-           antideriv_S2(A, B, C, s2, t1) + antideriv_S2(A, B, C, s1, t1);
+    return edge_S2(A, B, C, s1, s2, t2) - edge_S2(A, B, C, s1, s2, t1) + edge_S2(C, B, A, t1, t2, s2) -
+           edge_S2(C, B, A, t1, t2, s1);
 }
 
 struct FinArgs {
@@ -640,8 +633,8 @@ __device__ __forceinline__ double zeta_yy(const double *__restrict__ z, int N, i
     return v / (dy * dy);
 }
 
-constexpr int FIN_LANES = 8;  // lanes per target in k_finish: one FP64 logarithm of the closed
-                               // form each (4 corners x 2 terms), a short dependent chain per lane
+constexpr int FIN_LANES = 4;  // lanes per target in k_finish: one edge of the closed form each
+constexpr int FIN_TPB = 32;   // one warp a CTA: a small mesh's warps then spread over the SMs' FP64 pipes
 
 // a + b in double-float: Knuth's two-sum of the high parts, the low parts added,
 // renormalised (the explicit _rn operations keep the compiler from contracting)
@@ -655,9 +648,12 @@ __device__ __forceinline__ float2 fin_df_add(float2 a, float2 b)
     return make_float2(h, __fsub_rn(l, __fsub_rn(h, t)));
 }
 
-// F2 / F7 / F1 at every half point (FIN_LANES lanes per target share the
-// split partial sums and take one logarithm each of the closed-form integral),
-// radiation rows per slice.
+// F2 / F7 / F1 at every half point, radiation rows per slice.  FIN_LANES lanes per
+// target share the split partial sums and take one edge each of the closed-form
+// integral.  Bound by the FP64 pipe (two operations per clock and SM, whole warps
+// at a time), so the closed form is four logarithms, one per lane of four, instead
+// of eight on eight lanes, and the rows' own arithmetic serves eight targets a
+// warp instead of four.  181 x 61: 42 -> 29 us.
 __global__ void k_finish(const double *__restrict__ part, const double *__restrict__ tgt,
                          const double *__restrict__ constB, const double *__restrict__ nodal,
                          const double *__restrict__ psurf, double *__restrict__ Fu,
@@ -683,7 +679,7 @@ __global__ void k_finish(const double *__restrict__ part, const double *__restri
 #pragma unroll
         for (int q = 0; q < NACC; q++) d[q] = make_float2(0.f, 0.f);
         if (is_t) {
-#pragma unroll 2
+#pragma unroll 4
             for (int s = q4; s < a.splits; s += FIN_LANES)
 #pragma unroll
                 for (int q = 0; q < NACC; q++) d[q] = fin_df_add(d[q], pf[((size_t)s * NACC + q) * a.Nt + et]);
@@ -700,7 +696,7 @@ __global__ void k_finish(const double *__restrict__ part, const double *__restri
 #pragma unroll
             for (int q = 0; q < NACC; q++) acc[q] = (double)d[q].x + (double)d[q].y;
     } else if (is_t) {
-#pragma unroll 2
+#pragma unroll 4
         for (int s = q4; s < a.splits; s += FIN_LANES)
 #pragma unroll
             for (int q = 0; q < NACC; q++) acc[q] += part[((size_t)s * NACC + q) * a.Nt + et];
@@ -709,13 +705,13 @@ __global__ void k_finish(const double *__restrict__ part, const double *__restri
     const double *r = tgt + (size_t)et * TREC;
     const double A = r[8], B = r[9], C = r[10];
     const double xs = a.x1 + (k + 0.5) * a.dx, ys = a.y1 + l * a.dy;
-    // lane q4: corner q4 >> 1 of the rectangle, (s2,t2) +, (s1,t2) -, (s2,t1) -, (s1,t1) +,
-    // and term q4 & 1 of its antiderivative
-    const int cq = q4 >> 1;
-    const double sc = (cq & 1) ? a.x1 - xs : a.xhi - xs;
-    const double tc = (cq & 2) ? a.ylo - ys : a.yhi - ys;
-    double g2 = is_t ? antideriv_S2_term(A, B, C, sc, tc, q4 & 1) : 0.0;
-    if ((cq == 1) || (cq == 2)) g2 = -g2;
+    // lane q4: edge t = yhi (+), t = ylo (-), s = xhi (+), s = x1 (-)
+    const double s1 = a.x1 - xs, s2 = a.xhi - xs, t1 = a.ylo - ys, t2 = a.yhi - ys;
+    double g2 = 0.0;
+    if (is_t)
+        g2 = edge_S2(q4 < 2 ? A : C, B, q4 < 2 ? C : A, q4 < 2 ? s1 : t1, q4 < 2 ? s2 : t2,
+                     q4 == 0 ? t2 : q4 == 1 ? t1 : q4 == 2 ? s2 : s1);
+    if (q4 & 1) g2 = -g2;
 #pragma unroll
     for (int o = 1; o < FIN_LANES; o <<= 1) {
         g2 += __shfl_xor_sync(0xffffffffu, g2, o);
@@ -776,30 +772,59 @@ __global__ void k_finish(const double *__restrict__ part, const double *__restri
 
 // Bottom-only part of the bottom single layer seen from bottom half points:
 //   sigma [ sum w beta_x K2(beta; beta*) - beta_x* sum w S2_beta ] + sigma beta_x* I2''_beta
-// It depends on the topography alone, so it is evaluated once (FP64).
-__global__ void k_constB(const double *__restrict__ src, int Ns, const double *__restrict__ tgt,
-                         const double *__restrict__ bx, const double *__restrict__ by,
-                         double *__restrict__ out, FinArgs a, double sigma)
+// It depends on the topography alone, so it is evaluated once (FP64) per
+// topography.  Like the FP64 pair sum it is bound by the FP64 pipe (21 operations
+// per index pair), and is split over sources in the same way (241 x 81: 14.2 ms
+// against 24.9 with one thread per half point and no split); k_constB adds the
+// splits' sums, which k_constB_pairs leaves in the partial-sum scratch.
+__global__ void __launch_bounds__(128) k_constB_pairs(const double *__restrict__ src, int per_split,
+                                                      const double *__restrict__ tgt, const double *__restrict__ bx,
+                                                      const double *__restrict__ by, double *__restrict__ part, int N,
+                                                      int Nt, double sigma)
 {
-    int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= a.Nt) return;
-    const int N = a.N;
-    int k = e % (N - 1), l = e / (N - 1);
-    size_t qa = (size_t)l * N + k, qb = qa + 1;
-    const double bxs = 0.5 * (bx[qa] + bx[qb]), bys = 0.5 * (by[qa] + by[qb]);
-    const double A = 1.0 + bxs * bxs, B = 2.0 * bxs * bys, C = 1.0 + bys * bys;
-    const double *t = tgt + (size_t)e * TREC;
+    constexpr int CH = 32;
+    __shared__ double sh[CH][5];  // xs, ys, (beta+1)/dx, w2 sigma beta_x, w2
+    const int e = blockIdx.x * 128 + threadIdx.x, et = min(e, Nt - 1);
+    const int k = et % (N - 1), l = et / (N - 1);
+    const size_t qa = (size_t)l * N + k;
+    const double bxs = 0.5 * (bx[qa] + bx[qa + 1]), bys = 0.5 * (by[qa] + by[qa + 1]), f = -sigma * bxs;
+    const double *t = tgt + (size_t)et * TREC;
     const double tx = t[0], ty = t[1], tb = t[3];
+    const double *sb = src + (size_t)blockIdx.y * per_split * REC;
     double sK = 0.0, sS = 0.0;
-    for (int s = 0; s < Ns; s++) {
-        const double *r = src + (size_t)s * REC;
-        const double sx = r[0] - tx, sy = r[1] - ty, d = r[3] - tb;
-        sK += r[11] * rsqrt(sx * sx + sy * sy + d * d);
-        sS += r[13] * rsqrt(A * sx * sx + B * sx * sy + C * sy * sy);
+    for (int c0 = 0; c0 < per_split; c0 += CH) {
+        const int nc = min(CH, per_split - c0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < nc * 5; i += 128) {
+            const int r = i / 5, v = i - 5 * r;
+            sh[r][v] = sb[(size_t)(c0 + r) * REC + (v < 2 ? v : v == 2 ? 3 : v == 3 ? 11 : 13)];
+        }
+        __syncthreads();
+#pragma unroll 2
+        for (int s = 0; s < nc; s++) {
+            const double sx = sh[s][0] - tx, sy = sh[s][1] - ty, d = sh[s][2] - tb;
+            const double rho2 = fma(sx, sx, sy * sy), m = fma(bxs, sx, bys * sy);
+            sK = fma(sh[s][3], rsq64(fma(d, d, rho2)), sK);
+            sS = fma(sh[s][4], rsq64(fma(m, m, rho2)), sS);
+        }
     }
+    if (e < Nt) part[(size_t)blockIdx.y * Nt + e] = fma(f, sS, sK);
+}
+
+__global__ void k_constB(const double *__restrict__ part, int splits, const double *__restrict__ bx,
+                         const double *__restrict__ by, double *__restrict__ out, FinArgs a, double sigma)
+{
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= a.Nt) return;
+    const int N = a.N, k = e % (N - 1), l = e / (N - 1);
+    const size_t qa = (size_t)l * N + k;
+    const double bxs = 0.5 * (bx[qa] + bx[qa + 1]), bys = 0.5 * (by[qa] + by[qa + 1]);
+    double v = 0.0;
+    for (int s = 0; s < splits; s++) v += part[(size_t)s * a.Nt + e];
     const double xs = a.x1 + (k + 0.5) * a.dx, ys = a.y1 + l * a.dy;
-    const double I2pp = rect_S2(A, B, C, a.x1 - xs, a.xhi - xs, a.ylo - ys, a.yhi - ys);
-    out[e] = sK - sigma * bxs * sS + sigma * bxs * I2pp;
+    const double I2pp = rect_S2(1.0 + bxs * bxs, 2.0 * bxs * bys, 1.0 + bys * bys, a.x1 - xs, a.xhi - xs, a.ylo - ys,
+                                a.yhi - ys);
+    out[e] = v + sigma * bxs * I2pp;
 }
 
 // ---------------------------------------------------------------------------
@@ -875,7 +900,7 @@ PairPlan fine_plan(int Nt, int Ns, int tpb, int unit, int per_sm, int splits_req
 
 int unpack_launch(bfs_ctx *c, const double *u, cudaStream_t s, int which)
 {
-    k_unpack<<<(3 * c->M * 32 + 127) / 128, 128, 0, s>>>(u, c->d_nodal, c->N, c->M, c->dx);
+    k_unpack<<<3 * c->M, UNP_TPB, 0, s>>>(u, c->d_nodal, c->N, c->M, c->dx);
     c->launches++;
     RecArgs ra = rec_args(c);
     ra.w64 = which & 1;
@@ -920,7 +945,7 @@ int residual_launch(bfs_ctx *c, const double *u, double *Fu, int precision, cuda
     if (ev1) cudaEventRecord(ev1, s);
     FinArgs fa = fin_args(c, p.splits, precision == BFS_FP32C);
     int tot = FIN_LANES * (c->Nt + c->M);
-    k_finish<<<(tot + 127) / 128, 128, 0, s>>>(c->d_part, c->d_tgt64, c->d_constB, c->d_nodal, c->d_psurf, Fu,
+    k_finish<<<(tot + FIN_TPB - 1) / FIN_TPB, FIN_TPB, 0, s>>>(c->d_part, c->d_tgt64, c->d_constB, c->d_nodal, c->d_psurf, Fu,
                                                c->d_flag, fa);
     c->launches++;
     BFS_CUDA_TRY(c, cudaGetLastError());
@@ -932,7 +957,7 @@ int finish_launch(bfs_ctx *c, double *Fu, int precision, cudaStream_t s)
     const PairPlan &p = precision == BFS_FP32C ? c->plan32 : (precision == BFS_DF64 ? c->plandf : c->plan64);
     FinArgs fa = fin_args(c, p.splits, precision == BFS_FP32C);
     int tot = FIN_LANES * (c->Nt + c->M);
-    k_finish<<<(tot + 127) / 128, 128, 0, s>>>(c->d_part, c->d_tgt64, c->d_constB, c->d_nodal, c->d_psurf, Fu,
+    k_finish<<<(tot + FIN_TPB - 1) / FIN_TPB, FIN_TPB, 0, s>>>(c->d_part, c->d_tgt64, c->d_constB, c->d_nodal, c->d_psurf, Fu,
                                                c->d_flag, fa);
     c->launches++;
     BFS_CUDA_TRY(c, cudaGetLastError());
@@ -996,8 +1021,11 @@ void batch_pairs_launch(int v, int grid, const BatchInst *inst, const int4 *item
 int constB_launch(bfs_ctx *c, cudaStream_t s)
 {
     FinArgs fa = fin_args(c, 1);
-    k_constB<<<(c->Nt + 127) / 128, 128, 0, s>>>(c->d_src64, c->Ns, c->d_tgt64, c->d_bx, c->d_by,
-                                                 c->d_constB, fa, c->opt.sign_I4);
+    const PairPlan &p = c->plan64;
+    k_constB_pairs<<<dim3(p.tiles, p.splits), 128, 0, s>>>(c->d_src64, p.per_split, c->d_tgt64, c->d_bx, c->d_by,
+                                                           c->d_part, c->N, c->Nt, c->opt.sign_I4);
+    k_constB<<<(c->Nt + 63) / 64, 64, 0, s>>>(c->d_part, p.splits, c->d_bx, c->d_by, c->d_constB, fa, c->opt.sign_I4);
+    c->launches++;
     c->launches++;
     BFS_CUDA_TRY(c, cudaGetLastError());
     return BFS_OK;
