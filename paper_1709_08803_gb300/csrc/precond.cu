@@ -570,48 +570,50 @@ struct GemmBatch {
 
 constexpr int TM = 64, TN = 64, TK = 16;
 
+// FP64: bound by the FP64 pipe (two operations per clock and SM), so what counts
+// is an even share of it: 32 x 32 tiles (864 CTAs for the six products of a
+// 365-row slice; the 216 of 64 x 64 tiles left a third of the SMs idle in the
+// second wave).
+constexpr int DT = 32;
+
 __global__ void __launch_bounds__(256) k_dgemm(GemmBatch gb, int n, double alpha, double beta)
 {
-    __shared__ double As[TK][TM + 1];
-    __shared__ double Bs[TK][TN + 1];
+    __shared__ double As[TK][DT + 1];
+    __shared__ double Bs[TK][DT + 1];
     const double *A = gb.A[blockIdx.z], *B = gb.B[blockIdx.z];
     double *C = gb.C[blockIdx.z];
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    const int row0 = blockIdx.y * TM, col0 = blockIdx.x * TN;
-    double acc[4][4] = {};
+    const int row0 = blockIdx.y * DT, col0 = blockIdx.x * DT;
+    double acc[2][2] = {};
     for (int k0 = 0; k0 < n; k0 += TK) {
-        for (int e = threadIdx.x; e < TM * TK; e += 256) {
-            int r = e / TK, kk = e % TK;
-            int gr = row0 + r, gk = k0 + kk;
+#pragma unroll
+        for (int e = threadIdx.x; e < DT * TK; e += 256) {
+            const int r = e / TK, kk = e % TK, gr = row0 + r, gk = k0 + kk;
             As[kk][r] = (gr < n && gk < n) ? A[(size_t)gr * n + gk] : 0.0;
         }
-        for (int e = threadIdx.x; e < TK * TN; e += 256) {
-            int kk = e / TN, cc = e % TN;
-            int gk = k0 + kk, gc = col0 + cc;
+#pragma unroll
+        for (int e = threadIdx.x; e < TK * DT; e += 256) {
+            const int kk = e / DT, cc = e % DT, gk = k0 + kk, gc = col0 + cc;
             Bs[kk][cc] = (gk < n && gc < n) ? B[(size_t)gk * n + gc] : 0.0;
         }
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < TK; kk++) {
-            double a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; i++) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; j++) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-            for (int i = 0; i < 4; i++)
-#pragma unroll
-                for (int j = 0; j < 4; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+            const double a0 = As[kk][ty], a1 = As[kk][ty + 16], b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
+            acc[0][0] = fma(a0, b0, acc[0][0]);
+            acc[0][1] = fma(a0, b1, acc[0][1]);
+            acc[1][0] = fma(a1, b0, acc[1][0]);
+            acc[1][1] = fma(a1, b1, acc[1][1]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; i++) {
-        int gr = row0 + ty * 4 + i;
+    for (int i = 0; i < 2; i++) {
+        const int gr = row0 + ty + 16 * i;
         if (gr >= n) continue;
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            int gc = col0 + tx * 4 + j;
+        for (int j = 0; j < 2; j++) {
+            const int gc = col0 + tx + 16 * j;
             if (gc >= n) continue;
             double *cp = C + (size_t)gr * n + gc;
             *cp = beta == 0.0 ? alpha * acc[i][j] : fma(alpha, acc[i][j], beta * *cp);
@@ -1251,6 +1253,21 @@ __global__ void k_df2_split_inplace(double *x, size_t cnt)
     }
 }
 
+__global__ void k_eye(double *__restrict__ X, int n)
+{
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < (size_t)n * n; e += (size_t)gridDim.x * blockDim.x)
+        X[e] = e % (n + 1) == 0 ? 1.0 : 0.0;
+}
+
+// raises *flag if an entry of the residual R = I - D X is not small
+__global__ void k_check_residual(const double *__restrict__ R, int n, double bound, int *__restrict__ flag)
+{
+    bool bad = false;
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < (size_t)n * n; e += (size_t)gridDim.x * blockDim.x)
+        bad = bad || !(fabs(R[e]) <= bound);
+    if (bad) atomicOr(flag, 1);
+}
+
 // A^-1[k][j] = S[perm[k]][pinv[j]], from the hi/lo pairs into FP64
 __global__ void k_gjp_unperm(const float2 *__restrict__ S, const int *__restrict__ perm, double *__restrict__ D,
                              int n)
@@ -1275,7 +1292,8 @@ static int gemm_batch(bfs_ctx *c, std::vector<const double *> &A, std::vector<co
         GemmBatch gb;
         int cnt = (int)std::min<size_t>(GB_MAX, A.size() - o);
         for (int i = 0; i < cnt; i++) { gb.A[i] = A[o + i]; gb.B[i] = B[o + i]; gb.C[i] = C[o + i]; }
-        dim3 grid((nb + TN - 1) / TN, (nb + TM - 1) / TM, cnt);
+        const int t = df ? TM : DT;
+        dim3 grid((nb + t - 1) / t, (nb + t - 1) / t, cnt);
         if (df) k_dfgemm<<<grid, 256, 0, s>>>(gb, nb, alpha, beta);
         else k_dgemm<<<grid, 256, 0, s>>>(gb, nb, alpha, beta);
         c->launches++;
@@ -1678,7 +1696,18 @@ static size_t gj_data_doubles(int sms, int nmax)
     return std::max<size_t>(2 * (size_t)sms, 4 * (size_t)GJP_BMAX) * (size_t)nmax;
 }
 
+static int factor(bfs_ctx *c, int half_band, bool refined, bool &redo, cudaStream_t s);
+
 int precond_factor(bfs_ctx *c, int half_band, cudaStream_t s)
+{
+    bool redo = false;
+    const int rc = factor(c, half_band, true, redo, s);
+    return redo ? factor(c, half_band, false, redo, s) : rc;
+}
+
+// refined: FP64 factors may take their diagonal inverses from the double-float
+// kernels and one correction; redo is set when a slice's correction was too large.
+static int factor(bfs_ctx *c, int half_band, bool refined, bool &redo, cudaStream_t s)
 {
     int h = half_band >= 0 ? half_band : c->opt.half_band;
     if (h < 0) h = 0;
@@ -1743,6 +1772,7 @@ int precond_factor(bfs_ctx *c, int half_band, cudaStream_t s)
     double *tmp = c->d_gj + gj_doubles;
     // FP32 sweeps: blocked double-float inversions (FP64 ones otherwise)
     const bool df = c->opt.precond_precision == BFS_FP32C && c->opt.surface_tension == 0.0;
+    const bool refine = refined && !df && c->opt.surface_tension == 0.0 && nb >= 128;
     // D_k^-1 in place for the one or two diagonal blocks listed
     auto invert_diag = [&](const int *ks, int cnt) -> int {
         {  // rows in shared memory, no grid barrier
@@ -1753,6 +1783,32 @@ int precond_factor(bfs_ctx *c, int half_band, cudaStream_t s)
                 BFS_CUDA_TRY(c, cudaMemcpyAsync(work[i], dst[i], sizeof(double) * bsz, cudaMemcpyDeviceToDevice, s));
             }
             int r = df ? gj_panel_invert(c, work, dst, cnt, nb, s) : 1;
+            if (r == 1 && refine && cnt == 1) {
+                // FP64 from the double-float inverse X by one Newton-Schulz step, X + X R with
+                // R = I - D X, both products in FP64.  What X leaves in R (1e-6 at 365 rows)
+                // is 2^5 times the rounding an FP64 elimination would leave; the step squares R,
+                // so with |R_ij| <= 1 / (64 nb) the remainder nb |R|^2 is below half of that.
+                // A 365-row slice takes 0.9 ms against 3.4 in k_gj_rows, whose pivot columns each
+                // wait for an exchange between all CTAs (181 x 61: factorisation 320 -> 151 ms,
+                // error of an apply against 64 bits 1.6e-11 -> 6.9e-12).
+                double *D = c->d_gj + 2 * bsz, *X = c->d_gj + 3 * bsz, *R = c->d_gj + 4 * bsz;
+                BFS_CUDA_TRY(c, cudaMemcpyAsync(D, dst[0], sizeof(double) * bsz, cudaMemcpyDeviceToDevice, s));
+                r = gj_panel_invert(c, work, &X, 1, nb, s);
+                if (r < 0) return r;
+                if (r == 0) {
+                    std::vector<const double *> a{D}, b{X};
+                    std::vector<double *> o{R};
+                    k_eye<<<256, 256, 0, s>>>(R, nb);
+                    if ((r = gemm_batch(c, a, b, o, -1.0, 1.0, s))) return r;
+                    k_check_residual<<<256, 256, 0, s>>>(R, nb, 1.0 / (64.0 * nb), c->d_pivflag + 1);
+                    c->launches += 2;
+                    BFS_CUDA_TRY(c, cudaMemcpyAsync(dst[0], X, sizeof(double) * bsz, cudaMemcpyDeviceToDevice, s));
+                    a[0] = X;
+                    b[0] = R;
+                    o[0] = dst[0];
+                    return gemm_batch(c, a, b, o, 1.0, 1.0, s);
+                }
+            }
             if (r == 1) r = gj_rows_invert(c, work, dst, cnt, nb, s);
             if (r <= 0) return r;
         }
@@ -1889,10 +1945,14 @@ int precond_factor(bfs_ctx *c, int half_band, cudaStream_t s)
         }
     }
     c->pc_twist = twist;
-    int flag = 0;
-    BFS_CUDA_TRY(c, cudaMemcpyAsync(&flag, c->d_pivflag, sizeof(int), cudaMemcpyDeviceToHost, s));
+    int flags[2] = {0, 0};
+    BFS_CUDA_TRY(c, cudaMemcpyAsync(flags, c->d_pivflag, sizeof flags, cudaMemcpyDeviceToHost, s));
     BFS_CUDA_TRY(c, cudaStreamSynchronize(s));
-    if (flag) {
+    if (refine && (flags[0] || flags[1])) {
+        redo = true;
+        return BFS_OK;
+    }
+    if (flags[0]) {
         c->err = "zero pivot in a diagonal block of the preconditioner";
         return BFS_ESINGULAR;
     }
