@@ -182,6 +182,7 @@ struct bfs_ctx {
     int ldp32;                   // padded row length of d_pc32
     int flow_checked;
     double *d_gj;      // Gauss-Jordan work matrices and GEMM scratch
+    void *d_slices;    // operand slices of sg_gemm, while factoring
     void *d_gjscr;     // dataflow Gauss-Jordan: candidate slots, perm / pinv
     double *d_gjdata;  // dataflow Gauss-Jordan: candidate rows
     double *d_rowsum5; // Nt
@@ -229,6 +230,11 @@ extern const int kNumBatchVariants;
 int batch_pairs_occupancy(int v, int *blocks_per_sm);
 void batch_pairs_launch(int v, int grid, const BatchInst *inst, const int4 *items, int n_items,
                         unsigned int *counter, const unsigned char *mask, cudaStream_t s);
+
+// slice_gemm.cu
+void sg_alloc(bfs_ctx *c);
+int sg_gemm(bfs_ctx *c, const std::vector<const double *> &A, const std::vector<const double *> &B,
+            const std::vector<double *> &C, double alpha, double beta, cudaStream_t s);
 
 // condense.cu
 int cond_ok(const bfs_ctx *c);

@@ -570,10 +570,11 @@ struct GemmBatch {
 
 constexpr int TM = 64, TN = 64, TK = 16;
 
-// FP64: bound by the FP64 pipe (two operations per clock and SM), so what counts
-// is an even share of it: 32 x 32 tiles (864 CTAs for the six products of a
-// 365-row slice; the 216 of 64 x 64 tiles left a third of the SMs idle in the
-// second wave).
+// FP64 products of blocks below 128 rows, or with surface tension; the others are
+// slice_gemm.cu's.  Bound by the FP64 pipe (two operations per clock and SM), so
+// what counts is an even share of it: 32 x 32 tiles (six products of a 365-row
+// slice make 864 CTAs; the 216 of 64 x 64 tiles leave a third of the SMs idle in
+// the second wave: 1.65 against 1.85 ms for the products of such a slice).
 constexpr int DT = 32;
 
 __global__ void __launch_bounds__(256) k_dgemm(GemmBatch gb, int n, double alpha, double beta)
@@ -1286,6 +1287,7 @@ __global__ void k_gjp_unperm(const float2 *__restrict__ S, const int *__restrict
 static int gemm_batch(bfs_ctx *c, std::vector<const double *> &A, std::vector<const double *> &B,
                       std::vector<double *> &C, double alpha, double beta, cudaStream_t s)
 {
+    if (c->d_slices) return sg_gemm(c, A, B, C, alpha, beta, s);
     const int nb = c->nb;
     const bool df = c->opt.precond_precision == BFS_FP32C && c->opt.surface_tension == 0.0;
     for (size_t o = 0; o < A.size(); o += GB_MAX) {
@@ -1526,6 +1528,8 @@ void precond_free(bfs_ctx *c)
     c->sweep_ntags = 0;
     c->pc_twist = -1;
     cudaFree(c->d_gj);
+    cudaFree(c->d_slices);
+    c->d_slices = nullptr;
     cudaFree(c->d_gjscr);
     cudaFree(c->d_gjdata);
     c->d_gjscr = nullptr;
@@ -1736,6 +1740,7 @@ static int factor(bfs_ctx *c, int half_band, bool refined, bool &redo, cudaStrea
     const size_t gj_doubles = std::max<size_t>(8 * bsz, twist >= 0 ? 4 * (size_t)h * h * bsz : 0);
     // GEMM scratch: W and L of up to two eliminations at once (4 h blocks)
     BFS_CUDA_TRY(c, cudaMalloc(&c->d_gj, sizeof(double) * (gj_doubles + bsz * 4 * (size_t)(h > 0 ? h : 1))));
+    sg_alloc(c);
     BFS_CUDA_TRY(c, cudaMalloc(&c->d_rowsum5, sizeof(double) * (size_t)c->Nt));
     {  // dataflow Gauss-Jordan: 2 parities x CTAs of slots, 2 x (perm, pinv) of the largest
        // matrix, and 2 parities x CTAs candidate rows
@@ -1948,6 +1953,8 @@ static int factor(bfs_ctx *c, int half_band, bool refined, bool &redo, cudaStrea
     int flags[2] = {0, 0};
     BFS_CUDA_TRY(c, cudaMemcpyAsync(flags, c->d_pivflag, sizeof flags, cudaMemcpyDeviceToHost, s));
     BFS_CUDA_TRY(c, cudaStreamSynchronize(s));
+    cudaFree(c->d_slices);
+    c->d_slices = nullptr;
     if (refine && (flags[0] || flags[1])) {
         redo = true;
         return BFS_OK;
