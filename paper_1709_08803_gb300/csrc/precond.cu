@@ -574,7 +574,7 @@ constexpr int TM = 64, TN = 64, TK = 16;
 // slice_gemm.cu's.  Bound by the FP64 pipe (two operations per clock and SM), so
 // what counts is an even share of it: 32 x 32 tiles (six products of a 365-row
 // slice make 864 CTAs; the 216 of 64 x 64 tiles leave a third of the SMs idle in
-// the second wave: 1.65 against 1.85 ms for the products of such a slice).
+// the second wave: 17 products of such a slice take 1.65 ms, 15 took 1.85).
 constexpr int DT = 32;
 
 __global__ void __launch_bounds__(256) k_dgemm(GemmBatch gb, int n, double alpha, double beta)
@@ -985,15 +985,19 @@ __global__ void __launch_bounds__(GJP_TPB, 1) k_gjp_panel(GjPanelArgs a)
 
 // The same panel over a cluster of GJC_CS CTAs, rows split in contiguous
 // ranges, each range resident in its own CTA's shared memory, so that one
-// panel column costs 1/GJC_CS of the update in each CTA.  A pivot step has one
-// cluster barrier.  Before it, every CTA moves its rows' entries of column j
-// to fcol (zeroing them in S), picks its best unused row and copies that row,
-// its pivot entry and its key into a candidate slot of its own (two slots, by
-// column parity).  After it, every CTA reads the GJC_CS keys and the winner's
-// slot through distributed shared memory, forms 1/a and the scaled pivot row
-// itself (the same values in every CTA) and updates its rows.  The parity lets
-// a CTA publish column j+1 while slower ones still read column j; a final
-// cluster barrier keeps every CTA's shared memory alive until all reads end.
+// panel column costs 1/GJC_CS of the update in each CTA.  Bound by the latency of
+// the pivot exchange, so the update runs under it: as soon as the pivot row of
+// column j is known, every CTA takes its rows' entries of column j + 1 through the
+// update alone (to fcol, zeroed in S), picks its best unused row, and copies that
+// row as the update will leave it, its pivot entry and its key into a candidate
+// slot of its own (two slots, by column parity).  It arrives at the cluster
+// barrier, updates all its other entries for column j, and waits.  Then it reads
+// every CTA's slot through distributed shared memory in one go, takes the one
+// with the largest key and forms 1/a and the scaled pivot row itself (the same
+// values in every CTA).  A panel of 365 rows takes 110 us (122 with the update between
+// the barriers and two dependent remote reads).  The parity of slots, fcol and pr lets a CTA
+// publish column j + 1 while slower ones still read column j; a final cluster
+// barrier keeps every CTA's shared memory alive until all reads end.
 constexpr int GJC_CS = 8;
 
 struct GjcSlot {
@@ -1001,6 +1005,18 @@ struct GjcSlot {
     float2 piv;
     unsigned int key;
 };
+
+__device__ __forceinline__ void gjc_arrive()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void gjc_wait()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 
 template <int BW>
 __global__ void __cluster_dims__(GJC_CS, 1, 1) __launch_bounds__(GJP_TPB, 1) k_gjc_panel(GjPanelArgs a)
@@ -1011,7 +1027,7 @@ __global__ void __cluster_dims__(GJC_CS, 1, 1) __launch_bounds__(GJP_TPB, 1) k_g
     constexpr int RSTEP = GJP_WARPS * RPW;
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
-    extern __shared__ float2 ps[];  // S: chunk BW, fcol: chunk, pr: GJP_BMAX; then used: chunk bytes
+    extern __shared__ float2 ps[];  // S: chunk BW, fcol: 2 chunk, pr: 2 GJP_BMAX; then used: chunk bytes
     __shared__ GjcSlot slot[2];
     __shared__ unsigned int ck[GJP_WARPS];
     __shared__ int prow[GJP_BMAX];
@@ -1028,8 +1044,8 @@ __global__ void __cluster_dims__(GJC_CS, 1, 1) __launch_bounds__(GJP_TPB, 1) k_g
     float2 *Tm = mat ? a.T1 : a.T0;
     int *perm = a.perm + (size_t)mat * 2 * n;
     auto sx = [](int i, int c) { return (size_t)i * BW + (c ^ (i & (BW - 1))); };
-    float2 *S = ps, *fcol = ps + (size_t)chunk * BW, *pr = fcol + chunk;
-    unsigned char *used = reinterpret_cast<unsigned char *>(pr + GJP_BMAX);
+    float2 *S = ps, *fcol = ps + (size_t)chunk * BW, *pr = fcol + 2 * chunk;
+    unsigned char *used = reinterpret_cast<unsigned char *>(pr + 2 * GJP_BMAX);
     for (int i = tid; i < nr; i += GJP_TPB) used[i] = 0;
     __syncthreads();
     for (int q = tid; q < k0; q += GJP_TPB) {
@@ -1055,40 +1071,58 @@ __global__ void __cluster_dims__(GJC_CS, 1, 1) __launch_bounds__(GJP_TPB, 1) k_g
             }
     }
     __syncthreads();
+    // rows' entries of the next pivot column to fcol (zeroed in S), and this CTA's candidate
+    auto warp_key = [&](unsigned int key) {
+        key = __reduce_max_sync(0xffffffffu, key);
+        if (lane == 0) ck[warp] = key;
+    };
+    {
+        unsigned int key = 0;
+        for (int i = tid; i < nr; i += GJP_TPB) {
+            const float2 x = S[sx(i, 0)];
+            fcol[i] = x;
+            S[sx(i, 0)] = make_float2(0.f, 0.f);
+            if (!used[i]) key = max(key, gjp_key(x.x, rlo + i));
+        }
+        warp_key(key);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned int key = __reduce_max_sync(0xffffffffu, lane < GJP_WARPS ? ck[lane] : 0u);
+        if (key) {
+            const int li = (int)(GJP_ROWMASK - (key & GJP_ROWMASK)) - rlo;
+            for (int c = lane; c < bw; c += 32) slot[0].row[c] = S[sx(li, c)];
+            if (lane == 0) slot[0].piv = fcol[li];
+        }
+        if (lane == 0) slot[0].key = key;
+    }
+    gjc_arrive();
     for (int j = 0; j < bw; j++) {
         const int par = j & 1;
-        {  // column j out to fcol and zeroed; this CTA's candidate
-            unsigned int key = 0;
-            for (int i = tid; i < nr; i += GJP_TPB) {
-                const float2 x = S[sx(i, j)];
-                fcol[i] = x;
-                S[sx(i, j)] = make_float2(0.f, 0.f);
-                if (!used[i]) key = max(key, gjp_key(x.x, rlo + i));
-            }
-            key = __reduce_max_sync(0xffffffffu, key);
-            if (lane == 0) ck[warp] = key;
-        }
-        __syncthreads();
-        if (warp == 0) {  // the candidate slot: key, pivot entry and row (column j already zeroed)
-            const unsigned int key = __reduce_max_sync(0xffffffffu, lane < GJP_WARPS ? ck[lane] : 0u);
-            GjcSlot &sl = slot[par];
-            if (key) {
-                const int li = (int)(GJP_ROWMASK - (key & GJP_ROWMASK)) - rlo;
-                for (int c = lane; c < bw; c += 32) sl.row[c] = S[sx(li, c)];
-                if (lane == 0) sl.piv = fcol[li];
-            }
-            if (lane == 0) sl.key = key;
-        }
-        cluster.sync();
+        float2 *fc = fcol + par * chunk, *fn = fcol + (par ^ 1) * chunk, *pc = pr + par * GJP_BMAX;
+        gjc_wait();
         if (warp == 0) {  // the winner over the cluster, 1/a and the scaled pivot row
-            const unsigned int rk = lane < GJC_CS ? cluster.map_shared_rank(&slot[par], lane)->key : 0u;
+            // every CTA's candidate at once: one latency of distributed shared memory
+            const GjcSlot *ls = cluster.map_shared_rank(&slot[par], lane % GJC_CS);
+            const unsigned int rk = lane < GJC_CS ? ls->key : 0u;
+            float2 pv = ls->piv, rv[GJC_CS][NC];
+#pragma unroll
+            for (int r = 0; r < GJC_CS; r++)
+#pragma unroll
+                for (int c = 0; c < NC; c++) rv[r][c] = cluster.map_shared_rank(&slot[par], r)->row[cl + c * 32];
             const unsigned int wkey = __reduce_max_sync(0xffffffffu, rk);
-            const int w = __ffs(__ballot_sync(0xffffffffu, lane < GJC_CS && rk == wkey)) - 1;
-            const GjcSlot *ws = cluster.map_shared_rank(&slot[par], max(w, 0));
+            const int w = max(__ffs(__ballot_sync(0xffffffffu, lane < GJC_CS && rk == wkey)) - 1, 0);
             const int p = min((int)(GJP_ROWMASK - (wkey & GJP_ROWMASK)), n - 1);
-            const float2 piv = ws->piv;
+            const float2 piv = make_float2(__shfl_sync(0xffffffffu, pv.x, w), __shfl_sync(0xffffffffu, pv.y, w));
             const float2 inv = piv.x != 0.f ? df2_recip(piv) : make_float2(0.f, 0.f);
-            for (int c = lane; c < bw; c += 32) pr[c] = c == j ? inv : df2_mul(ws->row[c], inv);
+#pragma unroll
+            for (int c = 0; c < NC; c++) {
+                float2 v = rv[0][c];
+#pragma unroll
+                for (int r = 1; r < GJC_CS; r++) v = r == w ? rv[r][c] : v;
+                const int col = cl + c * 32;
+                if (col < bw) pc[col] = col == j ? inv : df2_mul(v, inv);
+            }
             if (lane == 0) {
                 if (piv.x == 0.f && rank == 0) atomicOr(a.pivflag, 1);
                 prow[j] = p;
@@ -1096,18 +1130,46 @@ __global__ void __cluster_dims__(GJC_CS, 1, 1) __launch_bounds__(GJP_TPB, 1) k_g
                 if (p >= rlo && p < rlo + nr) used[p - rlo] = 1;
             }
         }
-        __syncthreads();
-        // every row of this CTA: S[i][c] -= f_i pr[c]; then the pivot row takes pr
+        __syncthreads();  // pc, prow; and the update of column j - 1 is complete
         const int pl = prow[j] - rlo;
+        if (j + 1 < bw) {
+            const float2 pn = pc[j + 1];
+            unsigned int key = 0;
+            for (int i = tid; i < nr; i += GJP_TPB) {
+                const float2 x = i == pl ? pn : df2_fms(S[sx(i, j + 1)], fc[i], pn);
+                fn[i] = x;
+                S[sx(i, j + 1)] = make_float2(0.f, 0.f);
+                if (!used[i]) key = max(key, gjp_key(x.x, rlo + i));
+            }
+            warp_key(key);
+            __syncthreads();
+            if (warp == 0) {  // the candidate row as the update below will leave it
+                const unsigned int ky = __reduce_max_sync(0xffffffffu, lane < GJP_WARPS ? ck[lane] : 0u);
+                GjcSlot &sl = slot[par ^ 1];
+                if (ky) {
+                    const int li = (int)(GJP_ROWMASK - (ky & GJP_ROWMASK)) - rlo;
+                    const float2 f = fc[li];
+                    for (int c = lane; c < bw; c += 32)
+                        sl.row[c] = c == j + 1 ? make_float2(0.f, 0.f) : df2_fms(S[sx(li, c)], f, pc[c]);
+                    if (lane == 0) sl.piv = fn[li];
+                }
+                if (lane == 0) sl.key = ky;
+            }
+            __syncthreads();
+            gjc_arrive();
+        }
+        // every row of this CTA, column j + 1 excepted: S[i][c] -= f_i pr[c]; then the
+        // pivot row takes pr
         float2 prv[NC];
 #pragma unroll
-        for (int c = 0; c < NC; c++) prv[c] = cl + c * 32 < bw ? pr[cl + c * 32] : make_float2(0.f, 0.f);
+        for (int c = 0; c < NC; c++)
+            prv[c] = cl + c * 32 < bw && cl + c * 32 != j + 1 ? pc[cl + c * 32] : make_float2(0.f, 0.f);
         for (int q = 0; q < nfull; q += GJP_U) {
             float2 sv[GJP_U][NC], fv[GJP_U];
 #pragma unroll
             for (int u = 0; u < GJP_U; u++) {
                 const int i = r0 + (q + u) * RSTEP;
-                fv[u] = fcol[i];
+                fv[u] = fc[i];
 #pragma unroll
                 for (int c = 0; c < NC; c++) sv[u][c] = S[sx(i, cl + c * 32)];
             }
@@ -1124,7 +1186,7 @@ __global__ void __cluster_dims__(GJC_CS, 1, 1) __launch_bounds__(GJP_TPB, 1) k_g
         }
         for (int q = nfull; q < nrow; q++) {
             const int i = r0 + q * RSTEP;
-            const float2 f = fcol[i];
+            const float2 f = fc[i];
 #pragma unroll
             for (int c = 0; c < NC; c++) {
                 float2 *e = S + sx(i, cl + c * 32);
@@ -1134,8 +1196,8 @@ __global__ void __cluster_dims__(GJC_CS, 1, 1) __launch_bounds__(GJP_TPB, 1) k_g
         if (pl >= r0 && pl < nr && (pl - r0) % RSTEP == 0)
 #pragma unroll
             for (int c = 0; c < NC; c++) S[sx(pl, cl + c * 32)] = prv[c];
-        __syncthreads();
     }
+    __syncthreads();
     cluster.sync();  // no CTA leaves while another may still read its slots
     // E[:, P] out for this CTA's rows; the pivot rows jr = rank (mod GJC_CS) out
     // (panel columns: the identity), then zeroed with this CTA's panel columns
@@ -1628,7 +1690,7 @@ static int gj_panel_invert(bfs_ctx *c, double *const *work, double *const *dst, 
     // the cluster form (panels of 64, rows over GJC_CS CTAs) from 128 rows up,
     // when a cluster with its shared memory can be resident
     const int chunk = (n + GJC_CS - 1) / GJC_CS;
-    const size_t csmem = sizeof(float2) * ((size_t)chunk * 64 + chunk + GJP_BMAX) + (size_t)chunk;
+    const size_t csmem = sizeof(float2) * ((size_t)chunk * 64 + 2 * chunk + 2 * GJP_BMAX) + (size_t)chunk;
     bool clus = allow_cluster && n >= 128 && n <= (int)GJP_ROWMASK + 1 && csmem <= GJP_SMEM;
     if (clus) {
         clus = cudaFuncSetAttribute((const void *)k_gjc_panel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
