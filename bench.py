@@ -41,7 +41,14 @@ MUFU_PER_INDEX_PAIR = 5  # reciprocal square roots per (target, source) index pa
 PAIRS_TRAFFIC = 1.4336e6  # profiles/k_pairs_181x61.md (43 x 87 CTAs)
 # dram__bytes_read.sum + dram__bytes_write.sum of one FP32 sweep launch at
 # 181x61 from an ncu capture of the current kernel; None until captured
-APPLY_TRAFFIC = 500.9e6  # profiles/k_apply_sweep_181x61.md
+APPLY_TRAFFIC = None  # not captured since phi_x is eliminated from the blocks
+
+
+def _slice_rows(mesh, fp32):
+    """Rows of a slice block: phi_x is eliminated where csrc/condense.cu does so
+    (FP32 sweeps 140 to 256 columns, FP64 sweeps from 100)."""
+    cond = 140 <= mesh.N <= 256 if fp32 else mesh.N >= 100
+    return 2 * (mesh.N + 1) + 1 if cond else 3 * (mesh.N + 1)
 
 
 def _pc_prec(args):
@@ -303,7 +310,7 @@ def run_apply(args):
     ms = ev0.elapsed_time(ev1) / args.steps
     pinfo = ctx.precond_info()
     h = pinfo["half_band"]
-    nb = 3 * (mesh.N + 1)
+    nb = _slice_rows(mesh, args.precond == "fp32")
     blocks = sum(min(k, h) + 1 + min(mesh.M - 1 - k, h) for k in range(mesh.M))
     esz = 4 if args.precond == "fp32" else 8
     nbytes = blocks * nb * nb * esz + 6 * ctx.n * 8
@@ -678,7 +685,7 @@ def main():
     # slots), ahead of its 5 reciprocal square roots on the special-function
     # unit (16 lanes/clk/SM)
     achieved = FP32_OPS_PER_INDEX_PAIR * pairs_per_s / 1e12 if n32 else None
-    roofline_pairs = {"bound": "alu", "kernel": "k_pairs<float> (FP32C all-pairs quadrature, packed FP32x2)",
+    roofline_pairs = {"bound": "alu", "kernel": "k_pairs32 (FP32C all-pairs quadrature, packed FP32x2)",
                 "achieved": achieved, "peak": alu["ffma2_tops"], "unit": "T FP32 lane-ops/s",
                 "frac": (achieved / alu["ffma2_tops"]) if achieved else None,
                 # dram bytes read + written per launch, from an ncu capture of this kernel at 181x61
@@ -701,7 +708,7 @@ def main():
     # the preconditioner apply streams every stored factor block once (HBM-bound)
     pinfo = ctx.precond_info()
     h = pinfo["half_band"]
-    nb = 3 * (mesh.N + 1)
+    nb = _slice_rows(mesh, args.precond == "fp32")
     blocks = sum(min(k, h) + 1 + min(mesh.M - 1 - k, h) for k in range(mesh.M))
     esz = 4 if args.precond == "fp32" else 8
     apply_bytes = blocks * nb * nb * esz + 6 * ctx.n * 8

@@ -98,8 +98,9 @@ typedef struct {
     int outer_precision;  /* BFS_FP64 (default) or BFS_DF64 for the Newton residual
                              and the line search */
     int precond_precision; /* BFS_FP64 (default) or BFS_FP32C: storage and arithmetic
-                              of the preconditioner sweeps.  The factorisation is FP64
-                              either way; FP32C sweeps an FP32 copy of the factors
+                              of the preconditioner sweeps.  BFS_FP64 factors to FP64
+                              accuracy; FP32C factors to 48 bits (double-float) and
+                              sweeps an FP32 copy of the factors
                               (the preconditioner only steers GMRES, the Newton
                               residual and the converged u do not depend on it).
                               With surface_tension > 0 the sweeps stay FP64: the
@@ -215,8 +216,9 @@ int bfs_jvp(bfs_ctx *ctx, const double *u, const double *Fu, const double *z, do
 
 /* Forms the Jacobian of the linearised discrete system (Sec. 4.2, App. B),
    keeps the slice blocks within half_band of the diagonal (App. A), reorders
-   it slice by slice into 3(N+1) x 3(N+1) blocks and factors it by block LU
-   with partial pivoting inside each diagonal block.  Depends on the mesh, F
+   it slice by slice into 3(N+1) x 3(N+1) blocks (2(N+1)+1 rows where phi_x is
+   eliminated from every slice first) and factors it by block LU with partial
+   pivoting inside each diagonal block.  Depends on the mesh, F
    and n only.  half_band < 0 uses the option's value.  Synchronous.
    Errors: BFS_ESINGULAR, BFS_ENOMEM, BFS_ECUDA. */
 int bfs_precond_factor(bfs_ctx *ctx, int half_band, void *stream);

@@ -6,7 +6,9 @@
 // and the nb equations [F5, F6, F1(1..N-1) | F3, F4, F2 | F8, F9, F7].  P is then
 // an M x M block matrix of nb x nb blocks; App. A keeps the blocks within
 // half_band h of the diagonal, so block row l stores blocks l-h .. l+h at
-// d_pc + (l (2h+1) + (m - l + h)) nb^2 (row-major).
+// d_pc + (l (2h+1) + (m - l + h)) nb^2 (row-major).  Where condense.cu takes phi_x
+// out of the slices first, nb = 2(N+1)+1 and the blocks are formed there; the rest
+// of this file is the same.  Products of blocks from 128 rows up are slice_gemm.cu's.
 //
 // Entries (derived by differentiating the linear residual of App. B; every
 // kernel there is a function of horizontal distance only, and the linear
