@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(32 * (SW_ROWS + PW + 1), 1) k_apply_sweep(Flow
     __shared__ int abort_sh;
     __shared__ volatile int dead;
     __shared__ float outv[4][SW_ROWS];  // a task's rows, until the CTA's last warp stores them together
-    __shared__ int ndone;               // rows done since the launch
+    __shared__ int ndone[2];            // rows done in the even and in the odd tasks since the launch
     const float *pc = a.pc;
     const int nb = a.nb, NB = a.NB, h = a.h, nd = 2 * h + 1, ldp = a.ldp;
     const int nslot = a.nslot, rows = a.rows;
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(32 * (SW_ROWS + PW + 1), 1) k_apply_sweep(Flow
         abort_sh = (ld_tag(reinterpret_cast<const unsigned int *>(a.flag)) & 2u) != 0;
         tag_sh = ld_tag(a.tagp);
         dead = 0;
-        ndone = 0;
+        ndone[0] = ndone[1] = 0;
         for (int i = 0; i < nslot; i++) {
             mbar_init(&full[i], 1);
             mbar_init(&empty[i], nrv);
@@ -744,12 +744,14 @@ __global__ void __launch_bounds__(32 * (SW_ROWS + PW + 1), 1) k_apply_sweep(Flow
             alo[0] += ol;
         }
         // the CTA's rows go out in one store of its last warp: lines that many CTAs are
-        // about to poll are written once per CTA, not once per row
+        // about to poll are written once per CTA, not once per row.  A task without a
+        // critical block waits for task s - 2 only, so one warp may be done with task s + 1
+        // while another is still in task s: even and odd tasks have a counter each
         int last = 0;
         if (lane == 0) {
             outv[s & 3][warp] = acc[0] + alo[0];
             __threadfence_block();
-            last = atomicAdd(&ndone, 1) == nrv * (s + 1) - 1;
+            last = atomicAdd(&ndone[s & 1], 1) == nrv * ((s >> 1) + 1) - 1;
             mbar_arrive(&empty[slot]);  // every lane's reads of the slot came before the shuffles
         }
         if (__shfl_sync(0xffffffffu, last, 0)) {
