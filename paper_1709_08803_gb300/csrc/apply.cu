@@ -982,7 +982,9 @@ struct SweepShape {
 static bool sweep_shape(int nb, int h, int groups, int G, int ntask, SweepShape &S)
 {
     const int ldp = (nb + 3) / 4 * 4;
-    S.Gg = G / groups;  // CTAs of a group
+    // CTAs of a group: every one has a row at least, since a barrier of the kernel cannot
+    // be set up for no arrivals and only a CTA with rows is waited for by the others
+    S.Gg = std::min(G / groups, nb);
     S.bm = h + 1 <= 4 ? 4 : SW_BMAX;
     S.nq = ldp <= 384 ? 3 : 5;
     if (nb > 128 * S.nq || h + 1 > S.bm || S.Gg < 1) return false;

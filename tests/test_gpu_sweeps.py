@@ -54,3 +54,11 @@ def _check(N, M, h, half=0, repeats=0):
                                         (45, 16, 6, 0)])
 def test_overlapping_tasks(N, M, h, half):
     _check(N, M, h, half, repeats=2000)
+
+
+# Slices of fewer rows than a group has CTAs (15 to 141 rows, groups of 76 or 152): as many
+# CTAs as rows; 72 | 75 | 78 rows around a group of 76, 150 | 153 around one of 152.
+@pytest.mark.parametrize("N,M,h,half", [(4, 3, 0, 0), (4, 3, 1, 0), (10, 7, 0, 0), (10, 7, 2, 1), (23, 7, 1, 0), (24, 7, 1, 0),
+                                        (25, 7, 1, 0), (46, 5, 0, 0), (49, 5, 0, 0), (50, 5, 0, 0)])
+def test_fewer_rows_than_ctas(N, M, h, half):
+    _check(N, M, h, half, repeats=20)
