@@ -493,12 +493,18 @@ int cond_tables(bfs_ctx *c, cudaStream_t s)
     return BFS_OK;
 }
 
+// Shared memory of the kernels that stage rows of nodes: the limit of cond_fits,
+// asked for whatever a launch needs (without it their static arrays count towards
+// 48 KB too) and the same for every context.
+constexpr size_t COND_SMEM = 200 * 1024;
+
 int cond_form(bfs_ctx *c, cudaStream_t s)
 {
     const CondArgs a = cond_args(c);
+    for (const void *k : {(const void *)k_cond_form, (const void *)k_cond_scan<Cv32>, (const void *)k_cond_scan<Cv64>,
+                          (const void *)k_cond_conv<Cv32>, (const void *)k_cond_conv<Cv64>})
+        BFS_CUDA_TRY(c, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)COND_SMEM));
     const size_t sm = sizeof(double) * (4 * (size_t)c->N + 8);
-    if (sm > 48 * 1024)
-        BFS_CUDA_TRY(c, cudaFuncSetAttribute((const void *)k_cond_form, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     k_cond_form<<<dim3(c->N - 1, 2 * c->pc_h + 1, c->M), CF_TPB, sm, s>>>(a, c->d_pc, c->d_rowsum5);
     k_cond_form_rad<<<(c->M + 31) / 32, 32, 0, s>>>(a, c->d_pc);
     c->launches += 2;
@@ -522,7 +528,7 @@ static size_t conv_smem(const bfs_ctx *c, int h, size_t k, size_t g) { return (s
 int cond_fits(const bfs_ctx *c, int h)
 {
     if (c->opt.precond_precision == BFS_FP32C ? (c->N < 140 || c->N > 256) : c->N < 100) return 0;
-    return conv_smem(c, h, 8, 8) <= 200 * 1024 && sizeof(double) * (4 * (size_t)c->N + 8) <= 200 * 1024;
+    return conv_smem(c, h, 8, 8) <= COND_SMEM && sizeof(double) * (4 * (size_t)c->N + 8) <= COND_SMEM;
 }
 
 template <typename CV>
@@ -532,10 +538,6 @@ static int cond_pre_t(bfs_ctx *c, const double *r, const typename CV::K *k6, cud
     typename CV::G *g = reinterpret_cast<typename CV::G *>(c->d_zc + (size_t)c->M * c->nb);
     const size_t sm = conv_smem(c, c->pc_h, sizeof(typename CV::K), sizeof(typename CV::G));
     const size_t ss = sizeof(double) * (size_t)c->N;
-    if (sm > 48 * 1024)
-        BFS_CUDA_TRY(c, cudaFuncSetAttribute((const void *)k_cond_conv<CV>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    if (ss > 48 * 1024)
-        BFS_CUDA_TRY(c, cudaFuncSetAttribute((const void *)k_cond_scan<CV>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     k_cond_scan<CV><<<c->M, CS_TPB, ss, s>>>(a, r, g, c->d_rc);
     k_cond_conv<CV><<<dim3((c->N + 30) / 32, c->M), CC_TPB, sm, s>>>(a, r, k6, g, c->d_rc);
     c->launches += 2;
