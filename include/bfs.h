@@ -310,6 +310,9 @@ int bfs_sweep_schedule(int M, int half_band, int twisted, int *tasks_out, int ca
    sweeps and the task multiplies at least one block. */
 int bfs_debug_stall_sweep(bfs_ctx *ctx, int task);
 
+/* The same for the launch after `skip` (>= 0) direct ones that run as usual. */
+int bfs_debug_stall_later(bfs_ctx *ctx, int task, int skip);
+
 /* The inversions of the block factorisation (App. B: the inverted diagonal
    blocks D_k^-1 of the block LU, and the two-ended order's middle system) on
    caller matrices.  A: DEVICE, nmat (1 or 2) consecutive n x n row-major FP64

@@ -129,6 +129,7 @@ def lib():
         L.bfs_sweep_schedule.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, C(ctypes.c_int),
                                          ctypes.c_int, C(ctypes.c_int)]
         L.bfs_debug_stall_sweep.argtypes = [_VP, ctypes.c_int]
+        L.bfs_debug_stall_later.argtypes = [_VP, ctypes.c_int, ctypes.c_int]
         L.bfs_precond_info.argtypes = [_VP, C(ctypes.c_int)]
         L.bfs_solver_info.argtypes = [_VP, C(ctypes.c_int)]
         L.bfs_peak_probe.argtypes = [ctypes.c_int, ctypes.c_int, _VP, _VP, C(ctypes.c_double)]
@@ -266,10 +267,10 @@ class Context:
         return {"step_graphs": info[0], "conditional": info[1], "graphs_off": bool(info[2]),
                 "own_stream": bool(info[3])}
 
-    def debug_stall_sweep(self, task: int):
-        """Test hook: the next FP32 sweep launch waits in `task` for a vector no
-        task writes (its waits run out after the option wait_polls)."""
-        self._check(lib().bfs_debug_stall_sweep(self._ctx, int(task)))
+    def debug_stall_sweep(self, task: int, skip: int = 0):
+        """Test hook: the next FP32 sweep launch (after `skip` others) waits in `task`
+        for a vector no task writes (its waits run out after the option wait_polls)."""
+        self._check(lib().bfs_debug_stall_later(self._ctx, int(task), int(skip)))
 
     def solve(self, u, stream=None, raise_on_error: bool = True):
         st = bfs_stats()

@@ -1187,7 +1187,7 @@ int apply_flow_launch(bfs_ctx *c, const double *r, double *z, cudaStream_t s)
         if (rc) return rc;
     }
     // test hook: one wait of this launch is for a vector no task writes
-    const bool stall = c->sweep_table && c->dbg_stall_task >= 0 && !c->capturing;
+    const bool stall = c->sweep_table && c->dbg_stall_task >= 0 && !c->capturing && c->dbg_stall_skip-- == 0;
     if (stall) {
         std::vector<SweepDev> bad = c->h_tasks;
         SweepDev &t = bad[c->dbg_stall_task];
@@ -1240,18 +1240,21 @@ int bfs_sweep_schedule(int M, int half_band, int twisted, int *tasks_out, int ca
     return n;
 }
 
-int bfs_debug_stall_sweep(bfs_ctx *c, int task)
+int bfs_debug_stall_sweep(bfs_ctx *c, int task) { return bfs_debug_stall_later(c, task, 0); }
+
+int bfs_debug_stall_later(bfs_ctx *c, int task, int skip)
 {
     if (!c) return BFS_EINVAL;
     if (!c->pc_ready || !c->sweep_table) {
         c->err = "the stall hook needs the FP32 task-table sweeps";
         return BFS_EINVAL;
     }
-    if (task < 0 || task >= (int)c->h_tasks.size() || c->h_tasks[task].head.z == 0) {
+    if (skip < 0 || task < 0 || task >= (int)c->h_tasks.size() || c->h_tasks[task].head.z == 0) {
         c->err = "no waiting block in that task";
         return BFS_EINVAL;
     }
     c->dbg_stall_task = task;
+    c->dbg_stall_skip = skip;
     return BFS_OK;
 }
 

@@ -160,6 +160,7 @@ struct bfs_ctx {
     int flow_vs;                 // words of a slice of the tagged vectors
     size_t sweep_dyn;
     int dbg_stall_task;          // test hook: task whose first wait is made unsatisfiable, or -1
+    int dbg_stall_skip;          // sweep launches before that one
 
     // Arnoldi steps of bfs_solve replayed as CUDA graphs, one per (Krylov
     // index j, base residual buffer); cleared whenever a captured argument
@@ -258,6 +259,10 @@ struct Gm {
     State state;
 };
 double gm_last_eta(const bfs_options &o, double finf, double eta);
+constexpr double GM_EXTRA_ETA = 0.2;
+constexpr int GM_EXTRA_ITS = 12;
+bool gm_extra_step(const bfs_options &o, int k, double finf);
+int gm_extra_drop(bfs_ctx *c, cudaStream_t s);
 void gm_start(bfs_ctx *c, Gm &g, const double *u, const double *F, const double *Fbase,
               double fnorm2, double eta, int maxit, cudaStream_t s);
 void gm_cycle_begin(bfs_ctx *c, Gm &g, double beta, cudaStream_t s);

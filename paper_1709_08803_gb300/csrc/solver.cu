@@ -162,6 +162,29 @@ double gm_last_eta(const bfs_options &o, double finf, double eta)
     return std::min(eta, std::max(0.1 * o.tol / finf, 1e-3));
 }
 
+// An iterate that meets the tolerance (|F|_inf = finf <= tol, after k steps) by less than
+// a factor of five was mostly left there by the rounding of the Krylov products: with
+// Eisenstat-Walker terms one more step, to GM_EXTRA_ETA or GM_EXTRA_ITS Krylov iterations,
+// is taken from it.  The iterate stands where that step fails in any way or does not meet
+// the tolerance too.
+bool gm_extra_step(const bfs_options &o, int k, double finf)
+{
+    return o.forcing == 1 && o.krylov_precision != o.outer_precision && k > 0 && k < o.max_newton && finf > 0.2 * o.tol;
+}
+
+// After an extra step that failed: a timeout that it ran into is taken back together with
+// what it left half-way, since the call reports success and the next apply has to run.
+int gm_extra_drop(bfs_ctx *c, cudaStream_t s)
+{
+    int flag = 0;
+    BFS_CUDA_TRY(c, cudaMemcpyAsync(&flag, c->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+    BFS_CUDA_TRY(c, cudaStreamSynchronize(s));
+    if (!(flag & 2)) return BFS_OK;
+    BFS_CUDA_TRY(c, cudaMemsetAsync(c->d_flag, 0, sizeof(int), s));
+    BFS_CUDA_TRY(c, cudaMemsetAsync(c->d_tailbar, 0, 2 * sizeof(unsigned int), s));
+    return flow_reset(c, s);
+}
+
 void solver_axpby(bfs_ctx *c, double *y, const double *x, const double *z, double a, double b,
                   cudaStream_t s)
 {
@@ -1102,7 +1125,11 @@ static int solve_on(bfs_ctx *c, double *u, bfs_stats *st, cudaStream_t s)
     const double eta_min = c->opt.eta;
     double eta_k = c->opt.forcing == 1 ? std::max(eta_min, 0.1) : eta_min;
     double prev_f2 = -1.0, prev_lin = 0.0, last_mu = 0.0;
-    bool polish = false;  // one step from an iterate that already meets the tolerance
+    bool extra = false;  // one step from an iterate that already meets the tolerance
+    auto keep = [&]() {
+        const int r = gm_extra_drop(c, s);
+        return finish(r ? r : BFS_OK);
+    };
     for (int k = 0;; k++) {
         if (c->opt.forcing == 1 && prev_f2 > 0.0) {
             const double prev_eta = eta_k;
@@ -1129,15 +1156,9 @@ static int solve_on(bfs_ctx *c, double *u, bfs_stats *st, cudaStream_t s)
         S.fnorm_2 = f2;
         S.fnorm_inf = finf;
         if (!isfinite(f2) || !isfinite(finf)) return finish(BFS_ENAN);
-        // an iterate that meets the tolerance by less than a factor of five was mostly left
-        // there by the rounding of the Krylov products; with Eisenstat-Walker terms one
-        // more step, of at most 12 Krylov iterations, is taken from it, and the iterate
-        // stands where that step fails or does not meet the tolerance too
         if (finf <= c->opt.tol) {
-            if (polish || c->opt.forcing != 1 || c->opt.krylov_precision == outer || k == 0 ||
-                k >= c->opt.max_newton || finf <= 0.2 * c->opt.tol)
-                return finish(BFS_OK);
-            polish = true;
+            if (extra || !gm_extra_step(c->opt, k, finf)) return finish(BFS_OK);
+            extra = true;
         }
         const bool met = finf <= c->opt.tol;
         if (k >= c->opt.max_newton) return finish(BFS_ENOCONV);
@@ -1154,13 +1175,13 @@ static int solve_on(bfs_ctx *c, double *u, bfs_stats *st, cudaStream_t s)
         Gm gk{};
         gk.precs = g.precs;
         gk.jvs = g.jvs;
-        const double eta = met ? 0.2 : cur == outer ? gm_last_eta(c->opt, finf, eta_k) : eta_k;
-        gm_start(c, gk, u, c->d_F, Fbase, f2, eta, met ? std::min(12, c->opt.max_krylov) : c->opt.max_krylov, s);
+        const double eta = met ? GM_EXTRA_ETA : cur == outer ? gm_last_eta(c->opt, finf, eta_k) : eta_k;
+        gm_start(c, gk, u, c->d_F, Fbase, f2, eta, met ? std::min(GM_EXTRA_ITS, c->opt.max_krylov) : c->opt.max_krylov, s);
         rc = gmres(c, gk, s, f2);
         S.krylov_its += gk.its;
         g.precs = gk.precs;
         g.jvs = gk.jvs;
-        if (rc) return finish(met && rc != BFS_ECUDA ? BFS_OK : rc);
+        if (rc) return met && rc != BFS_ECUDA ? keep() : finish(rc);
         stalls = gk.res > gk.target ? stalls + 1 : 0;
         if (!met && c->opt.stall_newton > 0 && stalls >= c->opt.stall_newton) {
             c->err = "GMRES stalled above its tolerance in consecutive Newton steps";
@@ -1179,6 +1200,7 @@ static int solve_on(bfs_ctx *c, double *u, bfs_stats *st, cudaStream_t s)
             BFS_CUDA_TRY(c, cudaMemcpyAsync(hflag, c->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
             if ((rc = read_scalars(c, c->d_scal + 12, 2, s))) return finish(rc);
             if (*hflag & 2) {
+                if (met) return keep();
                 c->err = "a wait in the preconditioner sweeps timed out";
                 return finish(BFS_ETIMEOUT);
             }
@@ -1187,7 +1209,7 @@ static int solve_on(bfs_ctx *c, double *u, bfs_stats *st, cudaStream_t s)
                 ok = true;
                 break;
             }
-            if (met) return finish(BFS_OK);
+            if (met) return keep();
             mu *= 0.5;
         }
         if (!ok) {

@@ -1,0 +1,73 @@
+"""The step that a solve with Eisenstat-Walker terms takes from an iterate which
+meets the tolerance by less than a factor of five."""
+import numpy as np
+import pytest
+
+from paper_1709_08803_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1709_08803_gb300 import build
+    build.build()
+
+
+def _options(**kw):
+    from paper_1709_08803_gb300 import bfs
+    return bfs.default_options(krylov_precision=bfs.BFS_FP32C, outer_precision=bfs.BFS_DF64, eta=1e-2, refine_below=1e-5,
+                               precond_precision=bfs.BFS_FP32C, forcing=1, **kw)
+
+
+def _solve(problem, **kw):
+    """A solve with its steps launched one by one."""
+    from paper_1709_08803_gb300 import bfs
+    ctx = bfs.Context(*problem, _options(wait_polls=4000, **kw))
+    ctx.precond_factor()
+    ctx.profile_enable()
+    u = ctx.flat_guess()
+    return ctx, u, ctx.solve(u, raise_on_error=False)
+
+
+def _tolerance_with_extra_step(problem):
+    """A tolerance at which the last step is the extra one, and the solve without it
+    (the step limit one lower: an iterate at the limit is returned as it is)."""
+    for tol in np.geomspace(1e-6, 1e-11, 101):
+        _, _, st = _solve(problem, tol=tol)
+        if st["status"] == 0 and st["newton_its"] > 1:
+            ctx, u, before = _solve(problem, tol=tol, max_newton=st["newton_its"] - 1)
+            if before["status"] == 0:
+                assert 0.2 * tol < before["fnorm_inf"] <= tol
+                return tol, u, before, st
+    pytest.fail("no tolerance with an extra step")
+
+
+def test_timeout_in_the_extra_step():
+    """A sweep of the extra step times out: the iterate before it is returned with
+    BFS_OK, and the next apply runs."""
+    from paper_1709_08803_gb300 import bfs
+    problem = W.config_small_half()
+    tol, u0, before, st = _tolerance_with_extra_step(problem)
+    ctx = bfs.Context(*problem, _options(wait_polls=4000, tol=tol))
+    ctx.precond_factor()
+    r = torch.tensor(np.random.default_rng(3).standard_normal(ctx.n), device="cuda")
+    ref = ctx.precond_apply(r)
+    assert ctx.check_finite()
+    tbl, ntask = bfs.sweep_schedule(problem[0].M, ctx.precond_info()["half_band"], ctx.precond_info()["twist"] >= 0)
+    ctx.profile_enable()
+    ctx.debug_stall_sweep(int(np.flatnonzero(tbl[:, 2] > 0)[-1]), skip=before["precond_applies"])
+    u = ctx.flat_guess()
+    got = ctx.solve(u, raise_on_error=False)
+    assert got["status"] == bfs.BFS_OK
+    assert got["precond_applies"] > before["precond_applies"]  # the step was taken
+    assert got["newton_its"] == before["newton_its"] and got["fnorm_inf"] == before["fnorm_inf"]
+    assert torch.equal(u, u0)
+    z = torch.full_like(r, float("nan"))
+    ctx.precond_apply(r, out=z)
+    assert torch.equal(z, ref)
+    assert ctx.check_finite()
+    ctx.close()
