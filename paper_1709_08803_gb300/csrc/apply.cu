@@ -1127,8 +1127,9 @@ static unsigned int spin_limit(const bfs_ctx *c)
     return c->opt.wait_polls > 0 ? (unsigned int)c->opt.wait_polls : FL_SPIN;
 }
 
-// Returns 1 if launched, 0 if this apply is not for the FP32 sweep kernels
-// (FP64 sweeps, or slice blocks wider than their tiles), or a negative code.
+// Returns 1 if launched, 2 if launched with z written as float pairs, 0 if this apply is
+// not for the FP32 sweep kernels (FP64 sweeps, or slice blocks wider than their tiles),
+// or a negative code.
 int apply_flow_launch(bfs_ctx *c, const double *r, double *z, cudaStream_t s)
 {
     if (c->opt.precond_precision != BFS_FP32C || !c->d_pc32 || !c->d_flow) return 0;
@@ -1153,7 +1154,7 @@ int apply_flow_launch(bfs_ctx *c, const double *r, double *z, cudaStream_t s)
     a.ntags = c->sweep_ntags;
     a.nslot = c->sweep_nslot;
     a.rows = c->sweep_rows;
-    a.zpair = c->pc_cond;
+    a.zpair = c->sweep_table && c->pc_cond;
     FlowKernel kern;
     int tpb;
     size_t dyn = 0;
@@ -1209,7 +1210,7 @@ int apply_flow_launch(bfs_ctx *c, const double *r, double *z, cudaStream_t s)
     BFS_CUDA_TRY(c, e);
     c->launches++;
     c->flow_count++;
-    return 1;
+    return a.zpair ? 2 : 1;
 }
 
 }  // namespace bfs

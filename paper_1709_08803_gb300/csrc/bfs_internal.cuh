@@ -243,7 +243,7 @@ int cond_fits(const bfs_ctx *c, int h);
 int cond_tables(bfs_ctx *c, cudaStream_t s);
 int cond_form(bfs_ctx *c, cudaStream_t s);
 int cond_pre(bfs_ctx *c, const double *r, cudaStream_t s);
-int cond_post(bfs_ctx *c, const double *r, double *z, cudaStream_t s);
+int cond_post(bfs_ctx *c, const double *r, double *z, bool pairs, cudaStream_t s);
 
 // pairs_df64.cu
 PairPlan plan_df(int Nt, int Ns, int splits_req, int sms);

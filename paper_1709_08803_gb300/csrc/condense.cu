@@ -553,9 +553,9 @@ int cond_pre(bfs_ctx *c, const double *r, cudaStream_t s)
     return cond_pre_t<Cv64>(c, r, a.k6, s);
 }
 
-int cond_post(bfs_ctx *c, const double *r, double *z, cudaStream_t s)
+int cond_post(bfs_ctx *c, const double *r, double *z, bool pairs, cudaStream_t s)
 {
-    if (c->sweep_table) k_cond_post<true><<<c->M, CS_TPB, 0, s>>>(cond_args(c), r, c->d_zc, z);
+    if (pairs) k_cond_post<true><<<c->M, CS_TPB, 0, s>>>(cond_args(c), r, c->d_zc, z);
     else k_cond_post<false><<<c->M, CS_TPB, 0, s>>>(cond_args(c), r, c->d_zc, z);
     c->launches++;
     BFS_CUDA_TRY(c, cudaGetLastError());

@@ -2063,8 +2063,8 @@ int precond_apply(bfs_ctx *c, const double *r, double *z, cudaStream_t s)
     }
     const int split = apply_flow_launch(c, rhs, sol, s);
     if (split < 0) return split;
-    if (split == 1) {
-        if (c->pc_cond) rc = cond_post(c, r, z, s);
+    if (split > 0) {
+        if (c->pc_cond) rc = cond_post(c, r, z, split == 2, s);
         if (ev1) cudaEventRecord(ev1, s);
         return rc;
     }
@@ -2092,7 +2092,7 @@ int precond_apply(bfs_ctx *c, const double *r, double *z, cudaStream_t s)
     BFS_CUDA_TRY(c, cudaLaunchCooperativeKernel((const void *)k_apply_coop, dim3(c->apply_grid),
                                                 dim3(AP_TPB), args, 0, s));
     c->launches++;
-    if (c->pc_cond) rc = cond_post(c, r, z, s);
+    if (c->pc_cond) rc = cond_post(c, r, z, false, s);
     if (ev1) cudaEventRecord(ev1, s);
     return rc;
 }
