@@ -495,7 +495,7 @@ int bfs_batch_solve(bfs_batch *b, double *const *u, bfs_stats *st, void *stream)
         std::vector<int> ls;
         for (int i : act) {
             S[i].krylov_its += g[i].its;
-            stalls[i] = g[i].res > g[i].target ? stalls[i] + 1 : 0;
+            stalls[i] = g[i].res > eta[i] * f2[i] ? stalls[i] + 1 : 0;  // the forcing term, as in bfs_solve
             if (g[i].status != BFS_OK) status[i] = g[i].status;
             else if (o.stall_newton > 0 && stalls[i] >= o.stall_newton) status[i] = BFS_ENOCONV;
             else { ls.push_back(i); mu[i] = 1.0; }

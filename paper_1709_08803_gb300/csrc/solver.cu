@@ -1182,7 +1182,8 @@ static int solve_on(bfs_ctx *c, double *u, bfs_stats *st, cudaStream_t s)
         g.precs = gk.precs;
         g.jvs = gk.jvs;
         if (rc) return met && rc != BFS_ECUDA ? keep() : finish(rc);
-        stalls = gk.res > gk.target ? stalls + 1 : 0;
+        // a stall is against the forcing term, not what gm_last_eta asks for beyond it
+        stalls = gk.res > eta_k * f2 ? stalls + 1 : 0;
         if (!met && c->opt.stall_newton > 0 && stalls >= c->opt.stall_newton) {
             c->err = "GMRES stalled above its tolerance in consecutive Newton steps";
             return finish(BFS_ENOCONV);

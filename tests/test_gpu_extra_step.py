@@ -1,5 +1,6 @@
-"""The step that a solve with Eisenstat-Walker terms takes from an iterate which
-meets the tolerance by less than a factor of five."""
+"""What a solve with Eisenstat-Walker terms does near its tolerance: GMRES of the last
+step goes on to a tenth of it, and an iterate which meets it by less than a factor of
+five gets one more step."""
 import numpy as np
 import pytest
 
@@ -71,3 +72,23 @@ def test_timeout_in_the_extra_step():
     assert torch.equal(z, ref)
     assert ctx.check_finite()
     ctx.close()
+
+
+@pytest.mark.parametrize("batch", [0, 1])
+def test_stall_is_against_the_forcing_term(batch):
+    """A forcing term of 0.9 that three Krylov iterations reach in every step is no
+    stall, although the last steps ask for more than three iterations give."""
+    from paper_1709_08803_gb300 import bfs
+    mesh, topo, F = W.config_small_half()
+    o = bfs.default_options(tol=1e-8, krylov_precision=bfs.BFS_FP32C, outer_precision=bfs.BFS_DF64, eta=0.9,
+                            refine_below=1e-5, forcing=1, max_krylov=3, stall_newton=1, max_newton=200)
+    if batch:
+        b = bfs.Batch([mesh], [topo], [F], o)
+        rc, st = b.solve(b.flat_guesses())
+        assert rc == bfs.BFS_OK and st[0]["fnorm_inf"] <= 1e-8, st
+        b.close()
+    else:
+        ctx = bfs.Context(mesh, topo, F, o)
+        st = ctx.solve(ctx.flat_guess(), raise_on_error=False)
+        assert st["status"] == bfs.BFS_OK and st["fnorm_inf"] <= 1e-8, st
+        ctx.close()
