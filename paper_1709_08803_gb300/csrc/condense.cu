@@ -20,7 +20,7 @@
 // known part of phi) and k_cond_post recovers phi_x.
 //
 // Not with surface tension, whose curvature term couples the F1 rows of
-// neighbouring slices (cond_ok).
+// neighbouring slices, nor on coarse meshes at small F, where it costs digits (cond_ok).
 //
 // The mesh is uniform, so every kernel value depends on the column offset and the
 // row distance alone: tables of K5, K7, K6 (row distance x column offset) are
@@ -56,13 +56,21 @@ static CondArgs cond_args(const bfs_ctx *c)
 }
 
 // phi_x can be taken first: no term that couples the F1 rows of two slices,
-// and a pivot n - 2 x1/dx of the first two phi_x that is no smaller than its
-// own terms (it is x1/dx large on the truncated meshes of Sec. 3.1).
+// a pivot n - 2 x1/dx of the first two phi_x that is no smaller than its own terms
+// (it is x1/dx large on the truncated meshes of Sec. 3.1), and no growth of the
+// rounding errors.  The elimination adds multiples of 2 pi dx^2/F^2 of zeta, summed over
+// the slice's nodes, to blocks of the size of 2 pi, so what decides is N dx^2/F^2.
+// Error of an FP64 apply against 64 bits, condensed over full blocks: 1.0 to 1.1 up to
+// 60 (dx = 0.1, 0.3), 1.2 at 90 (dx = 0.3), 1.8 at 75 (dx = 3), 1.6 at 100 (dx = 0.1), 3 at
+// 150 and 13 at 900 (dx = 3).  FP32: 1.2e-7 at 181 x 61 up to 150, 1.8e-7 at 300, 4.1e-7 at
+// 900 (6e-8 with full blocks).
+constexpr double COND_GROWTH = 75.0;
 int cond_ok(const bfs_ctx *c)
 {
     const double g = c->x1 / c->dx, piv = c->opt.n_rad - 2.0 * g;
     return c->opt.surface_tension == 0.0 && isfinite(piv) && fabs(piv) >= 1.0 &&
-           fabs(piv) >= 0.5 * (fabs(c->opt.n_rad) + 2.0 * fabs(g));
+           fabs(piv) >= 0.5 * (fabs(c->opt.n_rad) + 2.0 * fabs(g)) &&
+           c->N * c->dx * c->dx <= COND_GROWTH * c->F * c->F;
 }
 
 // Kernel values at row distance r dy and column offset (o - (N-2) - 1/2) dx,

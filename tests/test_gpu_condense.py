@@ -4,7 +4,11 @@ import os
 import subprocess
 import sys
 
+import numpy as np
 import pytest
+
+import oracle as O
+from paper_1709_08803_gb300 import workloads as W
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -52,3 +56,25 @@ def test_first_launch_near_48_KB(N, M, h, prec):
     r = subprocess.run([sys.executable, "-c", FRESH, *map(str, (N, M, h, prec))], cwd=ROOT, capture_output=True, text=True,
                        timeout=600)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+def _apply(mesh, h, prec, F):
+    from paper_1709_08803_gb300 import bfs
+    ctx = bfs.Context(mesh, W.flat_topography(mesh), F, bfs.default_options(precond_precision=prec))
+    ctx.precond_factor(h)
+    r = np.random.default_rng(mesh.N).standard_normal(mesh.n_unknowns)
+    z = ctx.precond_apply(torch.tensor(r, dtype=torch.float64, device="cuda")).cpu().numpy()
+    assert ctx.check_finite()
+    ctx.close()
+    return O.jtilde(O.problem(mesh, F), half_band=h), r, z
+
+
+# Coarse meshes and small Froude numbers, N dx^2 / F^2 from 40 over 74 (condensed) and 75.1 to 2e6:
+# the tolerances of test_gpu_factor.py, 1e-9 |r| |P| for FP64 and P z within 5 % of r for FP32.
+@pytest.mark.parametrize("N,M,h,dx,F,prec", [
+    (110, 7, 2, 3.0, 0.1, 0), (110, 7, 2, 3.0, 0.02, 0), (110, 7, 2, 0.3, 0.02, 0), (150, 5, 1, 0.3, 0.02, 0),
+    (101, 7, 2, 1.0, 1.16, 0), (101, 7, 2, 1.0, 1.17, 0), (101, 7, 2, 1.0, 1.6, 0),
+    (150, 5, 1, 0.3, 0.1, 1), (150, 5, 1, 0.3, 0.3, 1), (150, 5, 1, 0.3, 0.58, 1)])
+def test_small_froude_and_coarse_mesh(N, M, h, dx, F, prec):
+    P, r, z = _apply(W.mesh_box(N, M, dx, dx * 7 / 6), h, prec, F)
+    assert np.abs(P @ z - r).max() <= (1e-9 * np.abs(P).max() if prec == 0 else 0.05) * np.abs(r).max()
