@@ -39,6 +39,10 @@ constexpr int TREC = 16;
 //   0 column  1 row  2 zeta*/dx  4 zeta*/dx + 1/dx  6 (beta*+1)/dx - 1/dx
 //   8 (beta*+1)/dx  10 f*  12 g*  14 zeta_x*  16 zeta_y* dy/dx  18,19 unused
 constexpr int DSRC = 24, DTGT = 20;
+// Heights of either sheet, in mesh cells, up to which the df64 pair kernel takes the
+// differences of two of them as they come (pairs_df64.cu); k_records raises d_flag[1]
+// where a node of the residual at hand is higher.
+constexpr double DF_HIGH = 16.0;
 
 // Accumulators written by the pair kernels, per split and target:
 //   0  double and single layers at top targets (top and bottom sheets)
@@ -121,7 +125,7 @@ struct bfs_ctx {
     double *d_part;                // max splits * NACC * Nt
     double *d_constB;              // Nt: bottom-only single-layer part at bottom targets
     double *d_psurf;               // NM applied surface pressure, or nullptr
-    int *d_flag;                   // non-finite flag
+    int *d_flag;                   // [0] non-finite and timeout flags; [1] DF_HIGH exceeded
     float *d_srcdf;                // Ns_cap * DSRC double-float source records
     float *d_tgtdf;                // Nt * DTGT double-float target records
     bfs::PairPlan plan64, plan32, plandf;

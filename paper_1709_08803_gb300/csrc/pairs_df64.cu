@@ -27,7 +27,12 @@
 //   - Double and single layer of a pairing share one accumulation,
 //     (t / r^2 + w zeta_x) / r.
 // Renormalisation is left out inside a term: a low part may reach about 2^-22 of
-// the operands its high part came from.  The three accumulators, whose low parts
+// the operands its high part came from, and products drop low times low part.  That
+// is too much for the difference of two heights of one sheet that are many cells high,
+// where little is left of the high parts: it is renormalised (2 % more operations)
+// where a height of the residual at hand exceeds DF_HIGH = 16 cells.  Largest error of
+// a term without | with it: 2e-14 | 1e-14 at a third of a cell, 4e-13 | 4e-14 at 3.5 cells,
+// 5e-12 | 4e-13 at 50, 1.3e-9 | 7e-12 at 512 (the last is the rounding of the heights).  The three accumulators, whose low parts
 // collect one rounding error per term, are renormalised every fourth source pair
 // (without that the 281 x 281 residual loses two bits).
 #include <math.h>
@@ -138,13 +143,17 @@ __device__ __forceinline__ df2 both2(const float *p) { return df2{f2_both(p[0]),
 constexpr int PDF_TPB = 128, PDF_CH = 64;
 
 // Records: source pairs interleaved (value v of sources 2i and 2i+1 side by
-// side), see DSRC in bfs_internal.cuh; targets DTGT floats each.
-template <bool SQ>
-__global__ void __launch_bounds__(PDF_TPB, 4)
-k_pairs_df(const float *__restrict__ src, int per_split, const float *__restrict__ tgt, int Nt,
-           double *__restrict__ part, float ry2h, float ry2l, double ry, double dy)
+// side), see DSRC in bfs_internal.cuh; targets DTGT floats each.  HIGH: heights beyond
+// DF_HIGH.
+template <bool SQ, bool HIGH>
+__device__ __forceinline__ void pair_tile_df(const float *__restrict__ src, int per_split, const float *__restrict__ tgt,
+                                             int Nt, double *__restrict__ part, float ry2h, float ry2l, double ry,
+                                             double dy, float *sh)
 {
-    __shared__ __align__(16) float sh[PDF_CH * DSRC];
+    auto diff = [](df2 a, df2 b) {
+        if constexpr (HIGH) return d2_norm(d2_sub(a, b));
+        else return d2_sub(a, b);
+    };
     const int split = blockIdx.y;
     const float *sb = src + (size_t)split * per_split * DSRC;
     const int t = blockIdx.x * PDF_TPB + threadIdx.x;
@@ -188,7 +197,7 @@ k_pairs_df(const float *__restrict__ src, int per_split, const float *__restrict
             const df2 zxd = val(18);
             // top target, top source: w (f - f*) K1 + w zeta_x K2
             {
-                const df2 d = d2_sub(zs, tz);
+                const df2 d = diff(zs, tz);
                 const Seed s = d2_seed(d2_r2<SQ>(rho2, d));
                 // w f - w f*: w is a power of two, so the product is exact
                 const f2 v = f2_fma(ntf.h, cw, w1f.h);
@@ -215,7 +224,7 @@ k_pairs_df(const float *__restrict__ src, int per_split, const float *__restrict
             }
             // bottom target, bottom source: -w (g - g*) K1(beta)
             {
-                const df2 d = d2_sub(bs, tB);
+                const df2 d = diff(bs, tB);
                 const Seed s = d2_seed(d2_r2<SQ>(rho2, d));
                 const f2 v = f2_fma(ntg.h, cw, w1g.h);
                 const f2 bb = f2_sub(v, w1g.h);
@@ -243,6 +252,16 @@ k_pairs_df(const float *__restrict__ src, int per_split, const float *__restrict
     }
 }
 
+template <bool SQ>
+__global__ void __launch_bounds__(PDF_TPB, 4)
+k_pairs_df(const float *__restrict__ src, int per_split, const float *__restrict__ tgt, int Nt,
+           double *__restrict__ part, float ry2h, float ry2l, double ry, double dy, const int *__restrict__ form)
+{
+    __shared__ __align__(16) float sh[PDF_CH * DSRC];
+    if (*form == 0) pair_tile_df<SQ, false>(src, per_split, tgt, Nt, part, ry2h, ry2l, ry, dy, sh);
+    else pair_tile_df<SQ, true>(src, per_split, tgt, Nt, part, ry2h, ry2l, ry, dy, sh);
+}
+
 PairPlan plan_df(int Nt, int Ns, int splits_req, int sms)
 {
     return fine_plan(Nt, Ns, PDF_TPB, 8, 5, splits_req, sms);
@@ -258,10 +277,10 @@ int pairs_df_launch(bfs_ctx *c, cudaStream_t s)
     const bool sq = c->dx == c->dy && c->N <= 1024 && c->M <= 512 && c->dx * 1024.0 >= 1.0;
     if (sq)
         k_pairs_df<true><<<grid, PDF_TPB, 0, s>>>(c->d_srcdf, p.per_split, c->d_tgtdf, c->Nt, c->d_part, ry2h,
-                                                  ry2l, ryd, c->dy);
+                                                  ry2l, ryd, c->dy, c->d_flag + 1);
     else
         k_pairs_df<false><<<grid, PDF_TPB, 0, s>>>(c->d_srcdf, p.per_split, c->d_tgtdf, c->Nt, c->d_part, ry2h,
-                                                   ry2l, ryd, c->dy);
+                                                   ry2l, ryd, c->dy, c->d_flag + 1);
     c->launches++;
     BFS_CUDA_TRY(c, cudaGetLastError());
     return BFS_OK;

@@ -27,8 +27,9 @@ namespace bfs {
 // and a short sum over the warps' totals, instead of a chain of passes in one warp.
 constexpr int UNP_TPB = 256;
 __global__ void __launch_bounds__(UNP_TPB) k_unpack(const double *__restrict__ u, double *__restrict__ nodal, int N,
-                                                    int M, double dx)
+                                                    int M, double dx, int *form)
 {
+    if (form && blockIdx.x == 0 && threadIdx.x == 0) *form = 0;  // of k_records
     __shared__ double tot[UNP_TPB / 32];
     const int f = blockIdx.x / M, j = blockIdx.x - f * M, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t NM = (size_t)N * M;
@@ -99,7 +100,7 @@ __global__ void __launch_bounds__(REC_TPB)
 k_records(double *nodal, const double *__restrict__ beta, const double *__restrict__ bx,
           const double *__restrict__ by, double *__restrict__ src64, float *__restrict__ src32,
           float *__restrict__ srcdf, double *__restrict__ tgt64, float *__restrict__ tgt32,
-          float *__restrict__ tgtdf, RecArgs a)
+          float *__restrict__ tgtdf, int *form, RecArgs a)
 {
     int e = blockIdx.x * blockDim.x + threadIdx.x;
     const int N = a.N, M = a.M;
@@ -166,6 +167,7 @@ k_records(double *nodal, const double *__restrict__ beta, const double *__restri
             for (int k = 0; k < 10; k++) split2(v[k], d[2 * (2 + 2 * k)], d[2 * (3 + 2 * k)]);
             d[44] = (float)c;
             d[46] = 0.f;
+            if (e < a.Ns && !(fabs(r[2]) <= DF_HIGH && fabs(r[3]) <= DF_HIGH)) *form = 1;  // every writer's value
         }
         return;
     }
@@ -900,7 +902,8 @@ PairPlan fine_plan(int Nt, int Ns, int tpb, int unit, int per_sm, int splits_req
 
 int unpack_launch(bfs_ctx *c, const double *u, cudaStream_t s, int which)
 {
-    k_unpack<<<3 * c->M, UNP_TPB, 0, s>>>(u, c->d_nodal, c->N, c->M, c->dx);
+    int *form = which & 4 ? c->d_flag + 1 : nullptr;
+    k_unpack<<<3 * c->M, UNP_TPB, 0, s>>>(u, c->d_nodal, c->N, c->M, c->dx, form);
     c->launches++;
     RecArgs ra = rec_args(c);
     ra.w64 = which & 1;
@@ -909,7 +912,7 @@ int unpack_launch(bfs_ctx *c, const double *u, cudaStream_t s, int which)
     int tot = c->Ns_cap + c->Nt;
     k_records<<<(tot + REC_TPB - 1) / REC_TPB, REC_TPB, 0, s>>>(c->d_nodal, c->d_beta, c->d_bx, c->d_by, c->d_src64,
                                                                 c->d_src32, c->d_srcdf, c->d_tgt64, c->d_tgt32,
-                                                                c->d_tgtdf, ra);
+                                                                c->d_tgtdf, form, ra);
     c->launches++;
     BFS_CUDA_TRY(c, cudaGetLastError());
     return BFS_OK;
