@@ -205,7 +205,7 @@ int bfs_setup(const bfs_mesh *mesh, const bfs_topo *topo, double F, const bfs_op
     ALLOC(c->d_tgtdf, sizeof(float) * bfs::DTGT * (size_t)c->Nt);
     ALLOC(c->d_part, sizeof(double) * c->part_cap);
     ALLOC(c->d_constB, sizeof(double) * (size_t)c->Nt);
-    ALLOC(c->d_flag, 2 * sizeof(int));
+    ALLOC(c->d_flag, 3 * sizeof(int));
     ALLOC(c->d_up, sizeof(double) * 2 * (size_t)c->n);
     c->d_Fp = c->d_up + c->n;
     ALLOC(c->d_scal, sizeof(double) * 32);

@@ -41,8 +41,9 @@ constexpr int TREC = 16;
 constexpr int DSRC = 24, DTGT = 20;
 // Heights of either sheet, in mesh cells, up to which the df64 pair kernel takes the
 // differences of two of them as they come (pairs_df64.cu); k_records raises d_flag[1]
-// where a node of the residual at hand is higher.
-constexpr double DF_HIGH = 16.0;
+// where a node of the residual at hand is higher.  DF_EXACT: vertical distances, in
+// cells, up to which its form for dx == dy is exact; d_flag[2] where one may be larger.
+constexpr double DF_HIGH = 16.0, DF_EXACT = 1447.0;
 
 // Accumulators written by the pair kernels, per split and target:
 //   0  double and single layers at top targets (top and bottom sheets)
@@ -125,7 +126,7 @@ struct bfs_ctx {
     double *d_part;                // max splits * NACC * Nt
     double *d_constB;              // Nt: bottom-only single-layer part at bottom targets
     double *d_psurf;               // NM applied surface pressure, or nullptr
-    int *d_flag;                   // [0] non-finite and timeout flags; [1] DF_HIGH exceeded
+    int *d_flag;                   // [0] non-finite and timeout flags; [1] DF_HIGH, [2] DF_EXACT exceeded
     float *d_srcdf;                // Ns_cap * DSRC double-float source records
     float *d_tgtdf;                // Nt * DTGT double-float target records
     bfs::PairPlan plan64, plan32, plandf;

@@ -86,7 +86,9 @@ __device__ __forceinline__ df2 d2_slope(df2 x, f2 s, df2 y, f2 t)
 
 // a = s^2 + t^2 + d^2.  SQ: rho2 is an exact multiple of 1/4, so rho2 - a.h is
 // exact (Sterbenz's lemma while d^2 <= rho2; beyond that both are multiples of
-// the spacing of a.h as long as a.h < 2^22) and one FMA gives the rest of d.h^2.
+// the spacing of a.h as long as a.h < 2^22, which |d| <= DF_EXACT ensures: a.h is then
+// at most 2 d^2) and one FMA gives the rest of d.h^2.  Past that a pair would be good to
+// about 2^-24 only.
 template <bool SQ>
 __device__ __forceinline__ df2 d2_r2(df2 rho2, df2 d)
 {
@@ -258,7 +260,8 @@ k_pairs_df(const float *__restrict__ src, int per_split, const float *__restrict
            double *__restrict__ part, float ry2h, float ry2l, double ry, double dy, const int *__restrict__ form)
 {
     __shared__ __align__(16) float sh[PDF_CH * DSRC];
-    if (*form == 0) pair_tile_df<SQ, false>(src, per_split, tgt, Nt, part, ry2h, ry2l, ry, dy, sh);
+    if (SQ && form[1]) pair_tile_df<false, true>(src, per_split, tgt, Nt, part, ry2h, ry2l, ry, dy, sh);
+    else if (form[0] == 0) pair_tile_df<SQ, false>(src, per_split, tgt, Nt, part, ry2h, ry2l, ry, dy, sh);
     else pair_tile_df<SQ, true>(src, per_split, tgt, Nt, part, ry2h, ry2l, ry, dy, sh);
 }
 
@@ -273,7 +276,8 @@ int pairs_df_launch(bfs_ctx *c, cudaStream_t s)
     const float ry2h = (float)ry2d, ry2l = (float)(ry2d - (double)ry2h);
     const PairPlan &p = c->plandf;
     const dim3 grid(p.tiles, p.splits);
-    // the exact-square form needs s^2 + t^2 and the depth within its exact range (d2_r2)
+    // the exact-square form needs s^2 + t^2 within its exact range, and vertical distances
+    // too (d2_r2): those are the data's, and the kernel leaves the form by d_flag[2]
     const bool sq = c->dx == c->dy && c->N <= 1024 && c->M <= 512 && c->dx * 1024.0 >= 1.0;
     if (sq)
         k_pairs_df<true><<<grid, PDF_TPB, 0, s>>>(c->d_srcdf, p.per_split, c->d_tgtdf, c->Nt, c->d_part, ry2h,

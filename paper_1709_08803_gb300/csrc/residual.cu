@@ -29,7 +29,7 @@ constexpr int UNP_TPB = 256;
 __global__ void __launch_bounds__(UNP_TPB) k_unpack(const double *__restrict__ u, double *__restrict__ nodal, int N,
                                                     int M, double dx, int *form)
 {
-    if (form && blockIdx.x == 0 && threadIdx.x == 0) *form = 0;  // of k_records
+    if (form && blockIdx.x == 0 && threadIdx.x == 0) form[0] = form[1] = 0;  // of k_records
     __shared__ double tot[UNP_TPB / 32];
     const int f = blockIdx.x / M, j = blockIdx.x - f * M, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t NM = (size_t)N * M;
@@ -167,7 +167,10 @@ k_records(double *nodal, const double *__restrict__ beta, const double *__restri
             for (int k = 0; k < 10; k++) split2(v[k], d[2 * (2 + 2 * k)], d[2 * (3 + 2 * k)]);
             d[44] = (float)c;
             d[46] = 0.f;
-            if (e < a.Ns && !(fabs(r[2]) <= DF_HIGH && fabs(r[3]) <= DF_HIGH)) *form = 1;  // every writer's value
+            // form: every writer's value is 1
+            const double lim = 0.5 * (DF_EXACT - a.idx);  // so that zeta, beta and 1/dx add up to DF_EXACT
+            if (e < a.Ns && !(fabs(r[2]) <= DF_HIGH && fabs(r[3]) <= DF_HIGH)) form[0] = 1;
+            if (e < a.Ns && !(fabs(r[2]) <= lim && fabs(r[3]) <= lim)) form[1] = 1;
         }
         return;
     }
@@ -210,6 +213,9 @@ k_records(double *nodal, const double *__restrict__ beta, const double *__restri
         o[1] = (float)r[15];
 #pragma unroll
         for (int k = 0; k < 8; k++) split2(v[k], o[2 + 2 * k], o[3 + 2 * k]);
+        // (zeta_x* s + zeta_y* t)^2 no larger than s^2 + t^2, or the sum within DF_EXACT
+        const double my = zys * a.ry, reach = fabs(zxs) * (N - 1) + fabs(my) * (a.half ? 2 * (M - 1) : M - 1);
+        if (!(zxs * zxs + my * my <= 0.99 || reach <= DF_EXACT)) form[1] = 1;
     }
 }
 
