@@ -131,9 +131,11 @@ typedef struct {
                               J s_{k-1}| | / |F_{k-1}|, safeguarded by eta_{k-1}^1.618
                               when that exceeds 0.1, kept in [eta, 0.9]; eta_0 =
                               max(eta, 0.1).  Where eta_k |F_k|_inf <= 5 tol the step
-                              goes on to 0.1 tol, and with a Krylov precision below the
-                              outer one an iterate between 0.2 tol and tol gets one
-                              more step of at most 12 Krylov iterations */
+                              goes on to 0.1 tol, and with another Krylov precision than
+                              the outer one bfs_solve (not bfs_batch_solve) takes one
+                              more step of at most 12 Krylov iterations from an iterate
+                              between 0.2 tol and tol; bfs_set_stop_at_tol turns both
+                              off */
     int wait_polls;        /* polls of a device-side wait (the tags of the preconditioner
                               sweeps, the grid barriers of the cooperative kernels) before
                               it gives up: the kernel raises the context's timeout bit,
@@ -191,6 +193,14 @@ int bfs_set_surface_pressure(bfs_ctx *ctx, const double *p);
    context unchanged, for F <= 0 or an F whose F^2/2 the current bottom
    reaches (the bound bfs_setup checks). */
 int bfs_set_froude(bfs_ctx *ctx, double F);
+
+/* on = 1: with Eisenstat-Walker terms (forcing = 1) a solve of ctx stops at the
+   first iterate with |F|_inf <= tol, and no GMRES is asked for more than its
+   forcing term.  0 (after bfs_setup): both go below tol as described there, which
+   takes the error of u that the rounding of the Krylov products leaves inside tol
+   down by 2 to 4, mostly for some Krylov iterations more (78 -> 90 at 181 x 61, F = 0.7).
+   For bfs_batch_solve, set it on every instance.  BFS_EINVAL for another value. */
+int bfs_set_stop_at_tol(bfs_ctx *ctx, int on);
 const char *bfs_last_error(const bfs_ctx *ctx);
 int bfs_n_unknowns(const bfs_ctx *ctx);
 /* Pair evaluations of one residual: 4 (N-1)M x (number of sources). */
@@ -371,7 +381,8 @@ int bfs_peak_probe_threads(void);
        and keeps the fastest (*ms_out: its batched-residual time).  Synchronous.
      bfs_batch_tuning: the chosen shape and the time of every candidate
        (ms_per_variant: 8 entries, -1 where not run).
-     bfs_batch_solve: bfs_solve for every instance, in lockstep (u: host array of
+     bfs_batch_solve: bfs_solve for every instance, without the step from an iterate that
+       meets tol (see forcing), in lockstep (u: host array of
        B device pointers; st: B stats or NULL).  Factors preconditioners that
        are not yet factored.  Synchronous.  Returns BFS_OK when every instance
        converged, otherwise the status of a failing instance (each instance's

@@ -122,6 +122,7 @@ def lib():
         L.bfs_bottom_pressure.argtypes = [_VP, _VP, _VP, C(ctypes.c_double), _VP]
         L.bfs_set_topography.argtypes = [_VP, C(bfs_topo)]
         L.bfs_set_froude.argtypes = [_VP, ctypes.c_double]
+        L.bfs_set_stop_at_tol.argtypes = [_VP, ctypes.c_int]
         L.bfs_set_surface_pressure.argtypes = [_VP, _VP]
         L.bfs_profile_enable.argtypes = [_VP, ctypes.c_int]
         L.bfs_profile_read.argtypes = [_VP, ctypes.POINTER(ctypes.c_double),
@@ -327,6 +328,10 @@ class Context:
     def set_froude(self, F: float):
         self._check(lib().bfs_set_froude(self._ctx, float(F)))
 
+    def set_stop_at_tol(self, on: bool = True):
+        """Solves with forcing = 1 stop at the first iterate that meets tol."""
+        self._check(lib().bfs_set_stop_at_tol(self._ctx, int(bool(on))))
+
     def profile_enable(self, on: bool = True):
         self._check(lib().bfs_profile_enable(self._ctx, int(bool(on))))
 
@@ -496,6 +501,11 @@ class Batch:
         self._check(lib().bfs_residual(lib().bfs_batch_instance(self._b, i), ctypes.c_void_p(_ptr(u)),
                                        ctypes.c_void_p(_ptr(out)), precision, _stream(stream)))
         return out
+
+    def set_stop_at_tol(self, on: bool = True):
+        """As Context.set_stop_at_tol, for every instance."""
+        for i in range(self.B):
+            self._check(lib().bfs_set_stop_at_tol(lib().bfs_batch_instance(self._b, i), int(bool(on))))
 
     def autotune(self, stream=None) -> float:
         ms = ctypes.c_double()

@@ -287,6 +287,14 @@ int bfs_set_froude(bfs_ctx *c, double F)
     return BFS_OK;
 }
 
+int bfs_set_stop_at_tol(bfs_ctx *c, int on)
+{
+    if (!c) return BFS_EINVAL;
+    if (on != 0 && on != 1) return set_err(c, BFS_EINVAL, "on must be 0 or 1");
+    c->stop_at_tol = on;
+    return BFS_OK;
+}
+
 void bfs_destroy(bfs_ctx *c)
 {
     if (!c) return;

@@ -453,7 +453,7 @@ int bfs_batch_solve(bfs_batch *b, double *const *u, bfs_stats *st, void *stream)
                 eta[i] = std::min(0.9, std::max(o.eta, e));
             }
             bfs::gm_start(c, g[i], u[i], c->d_F, cur[i] != o.krylov_precision ? c->d_F32 : c->d_F, f2[i],
-                          cur[i] == outer ? bfs::gm_last_eta(o, finf[i], eta[i]) : eta[i], o.max_krylov, s);
+                          cur[i] == outer ? bfs::gm_last_eta(c, finf[i], eta[i]) : eta[i], o.max_krylov, s);
         }
         if ((rc = read_batch(b, act, 8, 1, s))) return rc;
         for (int i : act) bfs::gm_cycle_begin(b->c[i], g[i], b->h_sc[4 * i], s);

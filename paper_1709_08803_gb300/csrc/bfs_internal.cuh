@@ -137,6 +137,7 @@ struct bfs_ctx {
     double *d_scal;       // 16 scalars
 
     // Newton / GMRES workspace
+    int stop_at_tol;  // bfs_set_stop_at_tol
     int m_alloc;
     double *d_V;      // (m+1) n Krylov basis
     double *d_Z;      // m n preconditioned basis vectors z_j = P^-1 v_j
@@ -263,10 +264,10 @@ struct Gm {
     int maxit, its, j, status, precs, jvs;
     State state;
 };
-double gm_last_eta(const bfs_options &o, double finf, double eta);
+double gm_last_eta(const bfs_ctx *c, double finf, double eta);
 constexpr double GM_EXTRA_ETA = 0.2;
 constexpr int GM_EXTRA_ITS = 12;
-bool gm_extra_step(const bfs_options &o, int k, double finf);
+bool gm_extra_step(const bfs_ctx *c, int k, double finf);
 int gm_extra_drop(bfs_ctx *c, cudaStream_t s);
 void gm_start(bfs_ctx *c, Gm &g, const double *u, const double *F, const double *Fbase,
               double fnorm2, double eta, int maxit, cudaStream_t s);

@@ -156,9 +156,10 @@ static int grid_for(int n) { return (n + 255) / 256 < 1184 ? (n + 255) / 256 : 1
 // the tolerance (no further than 1e-3 of |F|: FP32C products resolve no more).
 // Ending just above the tolerance costs another Newton step, ending just below it
 // leaves an iterate whose error is decided by where GMRES happened to stop.
-double gm_last_eta(const bfs_options &o, double finf, double eta)
+double gm_last_eta(const bfs_ctx *c, double finf, double eta)
 {
-    if (o.forcing != 1 || !(finf > 0.0) || eta * finf > 5.0 * o.tol) return eta;
+    const bfs_options &o = c->opt;
+    if (c->stop_at_tol || o.forcing != 1 || !(finf > 0.0) || eta * finf > 5.0 * o.tol) return eta;
     return std::min(eta, std::max(0.1 * o.tol / finf, 1e-3));
 }
 
@@ -167,9 +168,10 @@ double gm_last_eta(const bfs_options &o, double finf, double eta)
 // Eisenstat-Walker terms one more step, to GM_EXTRA_ETA or GM_EXTRA_ITS Krylov iterations,
 // is taken from it.  The iterate stands where that step fails in any way or does not meet
 // the tolerance too.
-bool gm_extra_step(const bfs_options &o, int k, double finf)
+bool gm_extra_step(const bfs_ctx *c, int k, double finf)
 {
-    return o.forcing == 1 && o.krylov_precision != o.outer_precision && k > 0 && k < o.max_newton && finf > 0.2 * o.tol;
+    const bfs_options &o = c->opt;
+    return !c->stop_at_tol && o.forcing == 1 && o.krylov_precision != o.outer_precision && k > 0 && k < o.max_newton && finf > 0.2 * o.tol;
 }
 
 // After an extra step that failed: a timeout that it ran into is taken back together with
@@ -1157,7 +1159,7 @@ static int solve_on(bfs_ctx *c, double *u, bfs_stats *st, cudaStream_t s)
         S.fnorm_inf = finf;
         if (!isfinite(f2) || !isfinite(finf)) return finish(BFS_ENAN);
         if (finf <= c->opt.tol) {
-            if (extra || !gm_extra_step(c->opt, k, finf)) return finish(BFS_OK);
+            if (extra || !gm_extra_step(c, k, finf)) return finish(BFS_OK);
             extra = true;
         }
         const bool met = finf <= c->opt.tol;
@@ -1175,7 +1177,7 @@ static int solve_on(bfs_ctx *c, double *u, bfs_stats *st, cudaStream_t s)
         Gm gk{};
         gk.precs = g.precs;
         gk.jvs = g.jvs;
-        const double eta = met ? GM_EXTRA_ETA : cur == outer ? gm_last_eta(c->opt, finf, eta_k) : eta_k;
+        const double eta = met ? GM_EXTRA_ETA : cur == outer ? gm_last_eta(c, finf, eta_k) : eta_k;
         gm_start(c, gk, u, c->d_F, Fbase, f2, eta, met ? std::min(GM_EXTRA_ITS, c->opt.max_krylov) : c->opt.max_krylov, s);
         rc = gmres(c, gk, s, f2);
         S.krylov_its += gk.its;

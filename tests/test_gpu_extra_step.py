@@ -92,3 +92,40 @@ def test_stall_is_against_the_forcing_term(batch):
         st = ctx.solve(ctx.flat_guess(), raise_on_error=False)
         assert st["status"] == bfs.BFS_OK and st["fnorm_inf"] <= 1e-8, st
         ctx.close()
+
+
+def _final(problem, batch, stop, **kw):
+    """Status and statistics of a solve, alone or as a batch of one."""
+    from paper_1709_08803_gb300 import bfs
+    mesh, topo, F = problem
+    if batch:
+        b = bfs.Batch([mesh], [topo], [F], _options(**kw))
+        b.set_stop_at_tol(stop)
+        _, st = b.solve(b.flat_guesses())
+        b.close()
+        return st[0]
+    ctx = bfs.Context(mesh, topo, F, _options(**kw))
+    ctx.set_stop_at_tol(stop)
+    st = ctx.solve(ctx.flat_guess(), raise_on_error=False)
+    ctx.close()
+    return st
+
+
+@pytest.mark.parametrize("batch", [0, 1])
+def test_stop_at_tol(batch):
+    """With it a solve never passes over an iterate that meets the tolerance, alone and in
+    a batch; without it, the solve alone takes the extra step for some of these tolerances."""
+    from paper_1709_08803_gb300 import bfs
+    problem = W.config_small_half()
+    passed = 0
+    for tol in np.geomspace(1e-7, 1e-11, 21):
+        for stop in (True, False):
+            st = _final(problem, batch, stop, tol=tol)
+            assert st["status"] == bfs.BFS_OK and st["fnorm_inf"] <= tol
+            short = _final(problem, batch, stop, tol=tol, max_newton=st["newton_its"] - 1)
+            assert short["status"] in (bfs.BFS_OK, bfs.BFS_ENOCONV)
+            if stop:
+                assert short["status"] == bfs.BFS_ENOCONV
+            else:
+                passed += short["status"] == bfs.BFS_OK
+    assert passed > 0 if not batch else passed == 0
