@@ -1455,11 +1455,11 @@ struct ApplyArgs {
 
 constexpr int AP_TPB = 1024;
 constexpr int AP_WARPS = AP_TPB / 32;
-constexpr int AP_NQ = 4;  // columns per lane and block row (a warp covers <= 128 columns)
+constexpr int AP_NQ = 4;  // columns per lane and block row and pass (a warp covers <= 128 columns)
 
 // One CTA per SM.  Rows of a slice are dealt out round-robin over the CTAs and
 // within a CTA over groups of warps; the warps of a group split the columns
-// of the row (at most 128 per warp, 4 per lane), and every lane first issues
+// of the row (at most 128 per warp and pass, 4 per lane), and every lane first issues
 // the loads of two blocks at once, so a step costs about two memory latencies
 // rather than one per column chunk.  Partial dots meet in shared memory.
 __global__ void __launch_bounds__(AP_TPB, 1) k_apply_coop(ApplyArgs a)
@@ -1518,7 +1518,8 @@ __global__ void __launch_bounds__(AP_TPB, 1) k_apply_coop(ApplyArgs a)
                 const int rr = rb + grp;
                 const int row = (grp < groups && rr < rpc) ? blockIdx.x + rr * gridDim.x : nb;
                 double acc = 0.0;
-                if (row < nb) {
+                // one pass up to 4096 columns, where a warp's are 128 at most
+                for (int cb = c0; cb < c1 && row < nb; cb += 32 * AP_NQ) {
                     for (int m = lo; m <= hi; m += 2) {
                         double fa[2][AP_NQ], va[2][AP_NQ];
 #pragma unroll
@@ -1529,7 +1530,7 @@ __global__ void __launch_bounds__(AP_TPB, 1) k_apply_coop(ApplyArgs a)
                             const double *v = (pass == 0 || mm == k) ? a.y + (size_t)mm * nb : a.x + (size_t)mm * nb;
 #pragma unroll
                             for (int q = 0; q < AP_NQ; q++) {
-                                const int c = c0 + lane + 32 * q;
+                                const int c = cb + lane + 32 * q;
                                 const bool in = ok && c < c1;
                                 fa[bb][q] = in ? __ldg(rp + c) : 0.0;
                                 va[bb][q] = in ? __ldcg(v + c) : 0.0;
