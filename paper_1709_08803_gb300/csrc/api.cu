@@ -39,13 +39,7 @@ void free_all(bfs_ctx *c)
     cudaFree(c->d_up);
     cudaFree(c->d_scal);
     cudaFree(c->d_red);
-    cudaFree(c->d_tailbar);
-    cudaFree(c->d_V);
-    cudaFree(c->d_Z);
-    cudaFree(c->d_H);
-    cudaFree(c->d_giv);
-    cudaFree(c->d_sbase);
-    if (c->h_pin) cudaFreeHost(c->h_pin);
+    bfs::free_solver(c);
     if (c->gm_ev) cudaEventDestroy(c->gm_ev);
     c->gm_ev = nullptr;
     if (c->join_ev) cudaEventDestroy(c->join_ev);

@@ -292,6 +292,7 @@ int jvp_launch(bfs_ctx *c, const double *u, const double *Fu, const double *z, d
 int solve_device(bfs_ctx *c, double *u, bfs_stats *st, cudaStream_t s);
 void gm_graphs_clear(bfs_ctx *c);
 int alloc_solver(bfs_ctx *c);
+void free_solver(bfs_ctx *c);
 void norms_launch(bfs_ctx *c, const double *v, int n, double *d_out2, double *d_outinf, cudaStream_t s);
 
 // precond.cu
@@ -352,6 +353,17 @@ __device__ __forceinline__ f2 f2_rsq(f2 x)
 }
 
 }  // namespace bfs
+
+// An allocation: no memory is BFS_ENOMEM, and not an error that the next launch would find.
+#define BFS_ALLOC_TRY(ctx, call)                                                     \
+    do {                                                                             \
+        cudaError_t e_ = (call);                                                     \
+        if (e_ != cudaSuccess) {                                                     \
+            cudaGetLastError();                                                      \
+            (ctx)->err = std::string(#call) + ": " + cudaGetErrorString(e_);         \
+            return e_ == cudaErrorMemoryAllocation ? BFS_ENOMEM : BFS_ECUDA;         \
+        }                                                                            \
+    } while (0)
 
 #define BFS_CUDA_TRY(ctx, call)                                                      \
     do {                                                                             \

@@ -470,24 +470,23 @@ __global__ void k_trisolve(const double *H, double *giv, int m, int k)
     }
 }
 
-int alloc_solver(bfs_ctx *c)
+static int alloc_solver_buffers(bfs_ctx *c)
 {
-    if (c->d_V) return BFS_OK;
     const int m = c->opt.gmres_restart, n = c->n;
     c->m_alloc = m;
-    BFS_CUDA_TRY(c, cudaMalloc(&c->d_V, sizeof(double) * (size_t)(m + 1) * n));
-    BFS_CUDA_TRY(c, cudaMalloc(&c->d_Z, sizeof(double) * (size_t)m * n));
-    BFS_CUDA_TRY(c, cudaMalloc(&c->d_H, sizeof(double) * (size_t)(m + 1) * m));
-    BFS_CUDA_TRY(c, cudaMalloc(&c->d_giv, sizeof(double) * (size_t)(6 * m + 4)));
-    BFS_CUDA_TRY(c, cudaMalloc(&c->d_sbase, sizeof(double) * (size_t)8 * n));
+    BFS_ALLOC_TRY(c, cudaMalloc(&c->d_V, sizeof(double) * (size_t)(m + 1) * n));
+    BFS_ALLOC_TRY(c, cudaMalloc(&c->d_Z, sizeof(double) * (size_t)m * n));
+    BFS_ALLOC_TRY(c, cudaMalloc(&c->d_H, sizeof(double) * (size_t)(m + 1) * m));
+    BFS_ALLOC_TRY(c, cudaMalloc(&c->d_giv, sizeof(double) * (size_t)(6 * m + 4)));
+    BFS_ALLOC_TRY(c, cudaMalloc(&c->d_sbase, sizeof(double) * (size_t)8 * n));
     double *b = c->d_sbase;
     c->d_F = b; c->d_du = b + n; c->d_ut = b + 2 * (size_t)n; c->d_Ft = b + 3 * (size_t)n;
     c->d_w = b + 5 * (size_t)n; c->d_F32 = b + 6 * (size_t)n;
     c->d_uio = b + 7 * (size_t)n;
-    BFS_CUDA_TRY(c, cudaMallocHost(&c->h_pin, sizeof(double) * 16));
+    BFS_ALLOC_TRY(c, cudaMallocHost(&c->h_pin, sizeof(double) * 16));
     // the fused Arnoldi tail: one CTA per SM (its partials, one per CTA and
     // dot, fit the reduction scratch of 32768 doubles for up to 128 dots)
-    BFS_CUDA_TRY(c, cudaMalloc(&c->d_tailbar, 2 * sizeof(unsigned int)));
+    BFS_ALLOC_TRY(c, cudaMalloc(&c->d_tailbar, 2 * sizeof(unsigned int)));
     BFS_CUDA_TRY(c, cudaMemset(c->d_tailbar, 0, 2 * sizeof(unsigned int)));
     {
         int per_sm = 0;
@@ -499,6 +498,30 @@ int alloc_solver(bfs_ctx *c)
             cudaGetLastError();
     }
     return BFS_OK;
+}
+
+// All of the solver's buffers or none: a failure gives back what it had got, so that a later
+// solve does not take the first of them for all.
+int alloc_solver(bfs_ctx *c)
+{
+    if (c->d_V) return BFS_OK;
+    const int rc = alloc_solver_buffers(c);
+    if (rc) free_solver(c);
+    return rc;
+}
+
+void free_solver(bfs_ctx *c)
+{
+    cudaFree(c->d_tailbar);
+    cudaFree(c->d_V);
+    cudaFree(c->d_Z);
+    cudaFree(c->d_H);
+    cudaFree(c->d_giv);
+    cudaFree(c->d_sbase);
+    if (c->h_pin) cudaFreeHost(c->h_pin);
+    c->d_tailbar = nullptr;
+    c->d_V = c->d_Z = c->d_H = c->d_giv = c->d_sbase = nullptr;
+    c->h_pin = nullptr;
 }
 
 static int read_scalars(bfs_ctx *c, const double *d, int cnt, cudaStream_t s)
