@@ -1097,7 +1097,7 @@ int precond_make_f32(bfs_ctx *c, cudaStream_t s)
     }
     if (table) {
         c->h_tasks = device_table(P, c->flow_vs, nv);
-        BFS_CUDA_TRY(c, cudaMalloc(&c->d_tasks, sizeof(SweepDev) * c->h_tasks.size()));
+        BFS_ALLOC_TRY(c, cudaMalloc(&c->d_tasks, sizeof(SweepDev) * c->h_tasks.size()));
         BFS_CUDA_TRY(c, cudaMemcpy(c->d_tasks, c->h_tasks.data(), sizeof(SweepDev) * c->h_tasks.size(),
                                    cudaMemcpyHostToDevice));
         c->sweep_table = 1;

@@ -481,22 +481,25 @@ __global__ void k_cond_cast(const double *__restrict__ x, float2 *__restrict__ y
         y[e] = cv_pack(x[e]);
 }
 
-// Tables, the row sums of w K5 into d_rowsum5 (before its closed-form part),
-// vectors of the reduced system.
+// Tables and the row sums of w K5 into d_rowsum5 (before its closed-form part); for
+// condensed blocks also K6 in float pairs and the vectors of the reduced system.
 int cond_tables(bfs_ctx *c, cudaStream_t s)
 {
     const int R = c->half ? 2 * c->M - 1 : c->M, ld = 2 * c->N - 2;
-    const size_t n = (size_t)R * ld, nv = (size_t)c->M * c->nb;
-    BFS_CUDA_TRY(c, cudaMalloc(&c->d_ktab, sizeof(double) * (4 * n + (size_t)R * (c->N - 1))));
-    BFS_CUDA_TRY(c, cudaMalloc(&c->d_rc, sizeof(double) * (2 * nv + (size_t)c->NM)));  // then phi of k_cond_scan
-    c->d_zc = c->d_rc + nv;
+    const size_t n = (size_t)R * ld, nv = (size_t)c->M * c->nb, nr = (size_t)R * (c->N - 1);
+    BFS_ALLOC_TRY(c, cudaMalloc(&c->d_ktab, sizeof(double) * ((c->pc_cond ? 4 : 3) * n + nr)));
     const CondArgs a = cond_args(c);
     double *rows = c->d_ktab + 3 * n;
     k_cond_tables<<<512, 256, 0, s>>>(a, c->d_ktab);
-    k_cond_cast<<<512, 256, 0, s>>>(a.k6, reinterpret_cast<float2 *>(rows + (size_t)R * (c->N - 1)), n);
+    if (c->pc_cond) {
+        BFS_ALLOC_TRY(c, cudaMalloc(&c->d_rc, sizeof(double) * (2 * nv + (size_t)c->NM)));  // then phi of k_cond_scan
+        c->d_zc = c->d_rc + nv;
+        k_cond_cast<<<512, 256, 0, s>>>(a.k6, reinterpret_cast<float2 *>(rows + nr), n);
+        c->launches++;
+    }
     k_cond_rows5<<<(R * (c->N - 1) + 7) / 8, 256, 0, s>>>(a, rows);
     k_cond_sum5<<<(c->Nt + 63) / 64, 64, 0, s>>>(a, rows, c->d_rowsum5);
-    c->launches += 4;
+    c->launches += 3;
     BFS_CUDA_TRY(c, cudaGetLastError());
     return BFS_OK;
 }

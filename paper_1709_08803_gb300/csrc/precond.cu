@@ -1770,8 +1770,10 @@ static int factor(bfs_ctx *c, int half_band, bool refined, bool &redo, cudaStrea
 int precond_factor(bfs_ctx *c, int half_band, cudaStream_t s)
 {
     bool redo = false;
-    const int rc = factor(c, half_band, true, redo, s);
-    return redo ? factor(c, half_band, false, redo, s) : rc;
+    int rc = factor(c, half_band, true, redo, s);
+    if (redo) rc = factor(c, half_band, false, redo, s);
+    if (rc == BFS_ENOMEM) precond_free(c);  // what it had got, back
+    return rc;
 }
 
 // refined: FP64 factors may take their diagonal inverses from the double-float
@@ -1804,18 +1806,18 @@ static int factor(bfs_ctx *c, int half_band, bool refined, bool &redo, cudaStrea
     // middle system; then h blocks of GEMM scratch
     const size_t gj_doubles = std::max<size_t>(8 * bsz, twist >= 0 ? 4 * (size_t)h * h * bsz : 0);
     // GEMM scratch: W and L of up to two eliminations at once (4 h blocks)
-    BFS_CUDA_TRY(c, cudaMalloc(&c->d_gj, sizeof(double) * (gj_doubles + bsz * 4 * (size_t)(h > 0 ? h : 1))));
+    BFS_ALLOC_TRY(c, cudaMalloc(&c->d_gj, sizeof(double) * (gj_doubles + bsz * 4 * (size_t)(h > 0 ? h : 1))));
     sg_alloc(c);
-    BFS_CUDA_TRY(c, cudaMalloc(&c->d_rowsum5, sizeof(double) * (size_t)c->Nt));
+    BFS_ALLOC_TRY(c, cudaMalloc(&c->d_rowsum5, sizeof(double) * (size_t)c->Nt));
     {  // dataflow Gauss-Jordan: 2 parities x CTAs of slots, 2 x (perm, pinv) of the largest
        // matrix, and 2 parities x CTAs candidate rows
         const int G = num_sms(c->device), nmax = std::max(nb, twist >= 0 ? h * nb : nb);
-        BFS_CUDA_TRY(c, cudaMalloc(&c->d_gjscr, sizeof(unsigned long long) * 4 * (size_t)G +
+        BFS_ALLOC_TRY(c, cudaMalloc(&c->d_gjscr, sizeof(unsigned long long) * 4 * (size_t)G +
                                                     sizeof(int) * 4 * (size_t)nmax));
-        BFS_CUDA_TRY(c, cudaMalloc(&c->d_gjdata, sizeof(double) * gj_data_doubles(G, nmax)));
+        BFS_ALLOC_TRY(c, cudaMalloc(&c->d_gjdata, sizeof(double) * gj_data_doubles(G, nmax)));
     }
-    BFS_CUDA_TRY(c, cudaMalloc(&c->d_pivflag, sizeof(int) * 8));  // [0] pivot flag, [4..5] grid barrier
-    BFS_CUDA_TRY(c, cudaMalloc(&c->d_perm_a, sizeof(double) * 2 * (size_t)c->n));
+    BFS_ALLOC_TRY(c, cudaMalloc(&c->d_pivflag, sizeof(int) * 8));  // [0] pivot flag, [4..5] grid barrier
+    BFS_ALLOC_TRY(c, cudaMalloc(&c->d_perm_a, sizeof(double) * 2 * (size_t)c->n));
     c->d_perm_b = c->d_perm_a + c->n;
     BFS_CUDA_TRY(c, cudaMemsetAsync(c->d_pc, 0, sizeof(double) * bsz * M * nd, s));
     BFS_CUDA_TRY(c, cudaMemsetAsync(c->d_pivflag, 0, sizeof(int) * 8, s));
@@ -2112,11 +2114,11 @@ extern "C" int bfs_gj_invert(const double *A, double *Ainv, int n, int nmat, int
     const size_t nn = (size_t)n * n;
     double *work = nullptr;
     auto run = [&]() -> int {
-        BFS_CUDA_TRY(c, cudaMalloc(&work, sizeof(double) * nmat * nn));
-        BFS_CUDA_TRY(c, cudaMalloc(&c->d_gjscr, sizeof(unsigned long long) * 4 * (size_t)G + sizeof(int) * 4 * (size_t)n));
-        BFS_CUDA_TRY(c, cudaMalloc(&c->d_gjdata, sizeof(double) * bfs::gj_data_doubles(G, n)));
-        BFS_CUDA_TRY(c, cudaMalloc(&c->d_pivflag, sizeof(int) * 8));
-        BFS_CUDA_TRY(c, cudaMalloc(&c->d_flag, sizeof(int)));
+        BFS_ALLOC_TRY(c, cudaMalloc(&work, sizeof(double) * nmat * nn));
+        BFS_ALLOC_TRY(c, cudaMalloc(&c->d_gjscr, sizeof(unsigned long long) * 4 * (size_t)G + sizeof(int) * 4 * (size_t)n));
+        BFS_ALLOC_TRY(c, cudaMalloc(&c->d_gjdata, sizeof(double) * bfs::gj_data_doubles(G, n)));
+        BFS_ALLOC_TRY(c, cudaMalloc(&c->d_pivflag, sizeof(int) * 8));
+        BFS_ALLOC_TRY(c, cudaMalloc(&c->d_flag, sizeof(int)));
         BFS_CUDA_TRY(c, cudaMemsetAsync(c->d_pivflag, 0, sizeof(int) * 8, s));
         BFS_CUDA_TRY(c, cudaMemsetAsync(c->d_flag, 0, sizeof(int), s));
         BFS_CUDA_TRY(c, cudaMemcpyAsync(work, A, sizeof(double) * nmat * nn, cudaMemcpyDeviceToDevice, s));

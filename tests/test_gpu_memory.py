@@ -50,3 +50,31 @@ def test_solver_buffers(leave):
             torch.cuda.empty_cache()
         assert ctx.solve(u)["status"] == bfs.BFS_OK
         ctx.close()
+
+
+# the factors (878 MB, 607 rows a slice and half band 1), then scratch (34 MB), then the
+# slices of the products (169 MB), without which other kernels take the products
+@pytest.mark.parametrize("leave,fits", [(500, 0), (890, 0), (960, 1)])
+def test_factor_buffers(leave, fits):
+    from paper_1709_08803_gb300 import bfs
+    ctx = _context()
+    ctx.precond_factor(1)
+    r = torch.randn(ctx.n, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    ref = ctx.precond_apply(r)
+    ctx.close()
+    ctx = _context()
+    hog = _leave(leave * MB)
+    if fits:
+        ctx.precond_factor(1)
+    else:
+        for _ in range(2):
+            with pytest.raises(bfs.BfsError) as e:
+                ctx.precond_factor(1)
+            assert e.value.code == bfs.BFS_ENOMEM
+    del hog
+    torch.cuda.empty_cache()
+    if not fits:
+        ctx.precond_factor(1)
+    # two factorisations to FP64 accuracy
+    assert (ctx.precond_apply(r) - ref).norm() <= 1e-9 * ref.norm()
+    ctx.close()
