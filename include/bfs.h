@@ -352,6 +352,10 @@ int bfs_gj_invert(const double *A, double *Ainv, int n, int nmat, int method, vo
 int bfs_profile_enable(bfs_ctx *ctx, int on);
 int bfs_profile_read(bfs_ctx *ctx, double *out8, unsigned long long *launches);
 
+/* Test hook: y[i] = 1/sqrt(x[i]), i < n, by the reciprocal root of the FP64 pair sum
+   (x, y: DEVICE).  Asynchronous on stream.  BFS_EINVAL for NULL or n < 1. */
+int bfs_rsqrt_probe(const double *x, double *y, int n, void *stream);
+
 /* Roofline probes (measurement only; the paper has no counterpart): one launch
    of a kernel that streams a single instruction kind through its pipe with
    no dependence between consecutive instructions and a full SM of warps:

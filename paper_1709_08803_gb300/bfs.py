@@ -122,6 +122,7 @@ def lib():
         L.bfs_bottom_pressure.argtypes = [_VP, _VP, _VP, C(ctypes.c_double), _VP]
         L.bfs_set_topography.argtypes = [_VP, C(bfs_topo)]
         L.bfs_set_froude.argtypes = [_VP, ctypes.c_double]
+        L.bfs_rsqrt_probe.argtypes = [_VP, _VP, ctypes.c_int, _VP]
         L.bfs_set_stop_at_tol.argtypes = [_VP, ctypes.c_int]
         L.bfs_set_surface_pressure.argtypes = [_VP, _VP]
         L.bfs_profile_enable.argtypes = [_VP, ctypes.c_int]
@@ -402,6 +403,16 @@ def peak_probe(kind: int, iters: int, out, stream=None) -> float:
     if rc:
         raise BfsError(rc, "peak probe failed")
     return ops.value
+
+
+def rsqrt_probe(x, stream=None):
+    """1/sqrt of the float64 CUDA vector x as the FP64 pair sum forms it."""
+    import torch
+    y = torch.empty_like(x)
+    rc = lib().bfs_rsqrt_probe(ctypes.c_void_p(_ptr(x)), ctypes.c_void_p(_ptr(y)), x.numel(), _stream(stream))
+    if rc:
+        raise BfsError(rc, "reciprocal root probe failed")
+    return y
 
 
 def gj_invert(A, method: int, stream=None):

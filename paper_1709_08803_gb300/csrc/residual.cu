@@ -228,7 +228,8 @@ k_records(double *nodal, const double *__restrict__ beta, const double *__restri
 // 2^-58).  Five FP64 instructions against the library call's eight, on a GPU
 // whose FP64 pipe retires two per clock and SM and bounds the FP64 pair sum.
 // a is at least 1/4 there (half-integer offsets in mesh units); an infinite a
-// gives 0 and a NaN gives NaN, as the library call does.
+// gives 0 and a NaN gives NaN, as the library call does.  Error below 1.6 2^-53: half
+// a unit of the last operation, 2^-54 from the rounding of a y.
 __device__ __forceinline__ double rsq64(double a)
 {
     double y;
@@ -236,6 +237,12 @@ __device__ __forceinline__ double rsq64(double a)
     double e = fma(-(a * y), y, 1.0);
     if (__double2hiint(a) == 0x7ff00000) e = 0.0;
     return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+__global__ void k_rsq64(const double *__restrict__ x, double *__restrict__ y, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) y[i] = rsq64(x[i]);
 }
 
 // Knuth's two-sum: hi + lo == a + b exactly.
@@ -1062,3 +1069,10 @@ void plans_for(int Nt, int Ns, int splits_req, int sms, PairPlan *p64, PairPlan 
 }
 
 }  // namespace bfs
+
+extern "C" int bfs_rsqrt_probe(const double *x, double *y, int n, void *stream)
+{
+    if (!x || !y || n < 1) return BFS_EINVAL;
+    bfs::k_rsq64<<<(n + 255) / 256, 256, 0, (cudaStream_t)stream>>>(x, y, n);
+    return cudaGetLastError() == cudaSuccess ? BFS_OK : BFS_ECUDA;
+}
