@@ -78,3 +78,65 @@ def _apply(mesh, h, prec, F):
 def test_small_froude_and_coarse_mesh(N, M, h, dx, F, prec):
     P, r, z = _apply(W.mesh_box(N, M, dx, dx * 7 / 6), h, prec, F)
     assert np.abs(P @ z - r).max() <= (1e-9 * np.abs(P).max() if prec == 0 else 0.05) * np.abs(r).max()
+
+
+# half domains (the images' terms), FP64: N dx^2 / F^2 = 18 to 21, so condensed
+@pytest.mark.parametrize("N,M,h", [(101, 7, 2), (102, 9, 3), (115, 6, 1)])
+def test_half_domain_fp64(N, M, h):
+    P, r, z = _apply(W.mesh_box(N, M, 0.3, 0.35, half=1), h, 0, 0.7)
+    assert np.abs(P @ z - r).max() <= 1e-9 * np.abs(r).max() * np.abs(P).max()
+
+
+# The FP32 sweeps against the FP64 ones: the relative errors stated with the kernels
+# (8.9e-8 at 151 x 53, 1.2e-7 at 181 x 61) times 5/3, which plain FP32 sums of the
+# eliminated unknowns exceed (2.8e-7 at 181 x 61).
+@pytest.mark.parametrize("N,M,bar", [(151, 53, 1.5e-7), (181, 61, 2.0e-7)])
+def test_fp32_sweeps_against_fp64(N, M, bar):
+    from paper_1709_08803_gb300 import bfs
+    mesh = W.mesh_box(N, M, 0.3, 0.3)
+    r = torch.tensor(np.random.default_rng(N).standard_normal(mesh.n_unknowns), device="cuda")
+    z = {}
+    for prec in (bfs.BFS_FP64, bfs.BFS_FP32C):
+        ctx = bfs.Context(mesh, W.flat_topography(mesh), 0.7, bfs.default_options(precond_precision=prec))
+        ctx.precond_factor()
+        z[prec] = ctx.precond_apply(r)
+        assert ctx.check_finite()
+        ctx.close()
+    assert (z[bfs.BFS_FP32C] - z[bfs.BFS_FP64]).norm() <= bar * z[bfs.BFS_FP64].norm()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_in_place_and_another_froude_number(prec):
+    """r may equal z, and the factors stay those of the Froude number they were formed for."""
+    from paper_1709_08803_gb300 import bfs
+    mesh = W.mesh_box(142, 9, 0.3, 0.3)
+    ctx = bfs.Context(mesh, W.flat_topography(mesh), 0.7, bfs.default_options(precond_precision=prec))
+    ctx.precond_factor(2)
+    r = torch.tensor(np.random.default_rng(1).standard_normal(mesh.n_unknowns), device="cuda")
+    z = ctx.precond_apply(r)
+    ctx.set_froude(0.9)
+    assert torch.equal(ctx.precond_apply(r), z)
+    x = r.clone()
+    ctx.precond_apply(x, out=x)
+    assert torch.equal(x, z)
+    assert ctx.check_finite()
+    ctx.close()
+
+
+def test_refused_inverse():
+    """Diagonal blocks that the double-float inverses are not good enough for are inverted
+    again in FP64: more launches, and the same bar."""
+    import ctypes
+    from paper_1709_08803_gb300 import bfs
+    mesh, launches = W.mesh_box(64, 5, 0.3, 0.3), {}
+    for F in (0.7, 1e-3):
+        ctx = bfs.Context(mesh, W.flat_topography(mesh), F)
+        n0, n1 = ctypes.c_ulonglong(), ctypes.c_ulonglong()
+        bfs.lib().bfs_profile_read(ctx._ctx, None, ctypes.byref(n0))
+        ctx.precond_factor(1)
+        bfs.lib().bfs_profile_read(ctx._ctx, None, ctypes.byref(n1))
+        launches[F] = n1.value - n0.value
+        ctx.close()
+    assert launches[1e-3] > launches[0.7]
+    P, r, z = _apply(mesh, 1, 0, 1e-3)
+    assert np.abs(P @ z - r).max() <= 1e-9 * np.abs(r).max() * np.abs(P).max()
