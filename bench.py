@@ -44,13 +44,6 @@ PAIRS_TRAFFIC = 1.4336e6  # profiles/k_pairs_181x61.md (43 x 87 CTAs)
 APPLY_TRAFFIC = None  # not captured since phi_x is eliminated from the blocks
 
 
-def _slice_rows(mesh, fp32):
-    """Rows of a slice block: phi_x is eliminated where csrc/condense.cu does so
-    (FP32 sweeps 140 to 256 columns, FP64 sweeps from 100)."""
-    cond = 140 <= mesh.N <= 256 if fp32 else mesh.N >= 100
-    return 2 * (mesh.N + 1) + 1 if cond else 3 * (mesh.N + 1)
-
-
 def _pc_prec(args):
     from paper_1709_08803_gb300 import bfs
     return bfs.BFS_FP32C if args.precond == "fp32" else bfs.BFS_FP64
@@ -310,7 +303,7 @@ def run_apply(args):
     ms = ev0.elapsed_time(ev1) / args.steps
     pinfo = ctx.precond_info()
     h = pinfo["half_band"]
-    nb = _slice_rows(mesh, args.precond == "fp32")
+    nb = pinfo["rows"]
     blocks = sum(min(k, h) + 1 + min(mesh.M - 1 - k, h) for k in range(mesh.M))
     esz = 4 if args.precond == "fp32" else 8
     nbytes = blocks * nb * nb * esz + 6 * ctx.n * 8
@@ -360,7 +353,7 @@ def run_factor(args):
     print(json.dumps({"mode": "factor", "metric": f"preconditioner factorisation at {mesh.N}x{mesh.M}",
                       "unit": "ms", "value": min(times), "mean_ms": sum(times) / len(times), "steps": args.steps,
                       "warmup": args.warmup, "half_band": pinfo["half_band"], "twist": pinfo["twist"],
-                      "precond": args.precond, "slice_block": 3 * (mesh.N + 1)}))
+                      "precond": args.precond, "slice_block": pinfo["rows"]}))
     ctx.close()
     return 0
 
@@ -708,7 +701,7 @@ def main():
     # the preconditioner apply streams every stored factor block once (HBM-bound)
     pinfo = ctx.precond_info()
     h = pinfo["half_band"]
-    nb = _slice_rows(mesh, args.precond == "fp32")
+    nb = pinfo["rows"]
     blocks = sum(min(k, h) + 1 + min(mesh.M - 1 - k, h) for k in range(mesh.M))
     esz = 4 if args.precond == "fp32" else 8
     apply_bytes = blocks * nb * nb * esz + 6 * ctx.n * 8

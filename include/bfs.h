@@ -240,6 +240,10 @@ int bfs_precond_factor(bfs_ctx *ctx, int half_band, void *stream);
    FP64 sweeps).  BFS_ENOPREC before bfs_precond_factor. */
 int bfs_precond_info(const bfs_ctx *ctx, int *info4);
 
+/* Rows of a factored slice block: 2(N+1)+1 where phi_x was eliminated from the
+   slices, else 3(N+1); BFS_ENOPREC before bfs_precond_factor. */
+int bfs_precond_rows(const bfs_ctx *ctx);
+
 /* How bfs_solve launched its Arnoldi steps (for tests and reports): info4[0]
    step graphs instantiated (one per Krylov index and base residual buffer,
    kept until a captured argument changes), info4[1] how many of them are

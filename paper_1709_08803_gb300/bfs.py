@@ -122,6 +122,7 @@ def lib():
         L.bfs_bottom_pressure.argtypes = [_VP, _VP, _VP, C(ctypes.c_double), _VP]
         L.bfs_set_topography.argtypes = [_VP, C(bfs_topo)]
         L.bfs_set_froude.argtypes = [_VP, ctypes.c_double]
+        L.bfs_precond_rows.argtypes = [_VP]
         L.bfs_rsqrt_probe.argtypes = [_VP, _VP, ctypes.c_int, _VP]
         L.bfs_set_stop_at_tol.argtypes = [_VP, ctypes.c_int]
         L.bfs_set_surface_pressure.argtypes = [_VP, _VP]
@@ -254,11 +255,13 @@ class Context:
         return out
 
     def precond_info(self) -> dict:
-        """Half band, two-ended split (-1: one-ended), sweep chains and the
-        dependent steps of the longest chain of the factored preconditioner."""
+        """Half band, two-ended split (-1: one-ended), sweep chains, the dependent
+        steps of the longest chain and the rows of a slice block of the factored
+        preconditioner."""
         info = (ctypes.c_int * 4)()
         self._check(lib().bfs_precond_info(self._ctx, info))
-        return {"half_band": info[0], "twist": info[1], "chains": info[2], "sweep_steps": info[3]}
+        return {"half_band": info[0], "twist": info[1], "chains": info[2], "sweep_steps": info[3],
+                "rows": lib().bfs_precond_rows(self._ctx)}
 
     def solver_info(self) -> dict:
         """How the solves of this context launched their Arnoldi steps: step

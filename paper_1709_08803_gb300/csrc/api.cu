@@ -350,6 +350,12 @@ int bfs_precond_info(const bfs_ctx *c, int *info)
     return BFS_OK;
 }
 
+int bfs_precond_rows(const bfs_ctx *c)
+{
+    if (!c) return BFS_EINVAL;
+    return c->pc_ready ? c->nb : BFS_ENOPREC;
+}
+
 int bfs_solver_info(const bfs_ctx *c, int *info)
 {
     if (!c || !info) return BFS_EINVAL;

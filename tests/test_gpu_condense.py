@@ -65,6 +65,9 @@ def _apply(mesh, h, prec, F):
     r = np.random.default_rng(mesh.N).standard_normal(mesh.n_unknowns)
     z = ctx.precond_apply(torch.tensor(r, dtype=torch.float64, device="cuda")).cpu().numpy()
     assert ctx.check_finite()
+    wide = mesh.N >= 100 if prec == 0 else 140 <= mesh.N <= 256
+    condensed = wide and mesh.N * mesh.dx ** 2 <= 75 * F ** 2
+    assert ctx.precond_info()["rows"] == (2 * mesh.N + 3 if condensed else 3 * mesh.N + 3)
     ctx.close()
     return O.jtilde(O.problem(mesh, F), half_band=h), r, z
 
