@@ -379,15 +379,30 @@ int sms()
     return bfs::num_sms(dev);
 }
 
-// both kernels stay below 48 KB of shared memory (dilation 27, 32 channels: 47.7 KB)
-size_t rows_smem(int C, int dil) { return (size_t)3 * (XS + 2 * dil) * C * 2; }
+constexpr size_t rows_smem(int C, int dil) { return (size_t)3 * (XS + 2 * dil) * C * 2; }
+constexpr size_t conv_smem(int C, int N, int dil) { return (size_t)N * (9 * C + 8) * 2 + rows_smem(C, dil); }
+constexpr size_t wgrad_smem(int C, int N, int dil) { return (size_t)XS * N * 2 + rows_smem(C, dil); }
+
+// Both kernels of every layer, each way, stay within the 48 KB of shared memory that a launch
+// may ask for without more (the largest is the convolution of 32 -> 32 channels at
+// dilation 9, 40.8 KB).
+constexpr size_t largest_smem()
+{
+    size_t m = 0;
+    for (int l = 0; l < NL; l++)
+        for (size_t b : {conv_smem(CIN[l], COUT[l], DIL[l]), conv_smem(COUT[l], CIN[l], DIL[l]),
+                         wgrad_smem(CIN[l], COUT[l], DIL[l])})
+            m = b > m ? b : m;
+    return m;
+}
+static_assert(largest_smem() <= 48 * 1024, "shared memory of the convolutions");
 
 template <int C, int N, int OUT>
 void conv(const __nv_bfloat16 *in, const __nv_bfloat16 *w, const float *b, float *z, __nv_bfloat16 *a, int Bt, int H,
           int W, int dil, int sgn, cudaStream_t s)
 {
     const int items = Bt * H * ((W + XS - 1) / XS);
-    k_conv<C, N, OUT><<<std::min(items, 4 * sms()), 2 * XS, N * (9 * C + 8) * 2 + rows_smem(C, dil), s>>>(
+    k_conv<C, N, OUT><<<std::min(items, 4 * sms()), 2 * XS, conv_smem(C, N, dil), s>>>(
         in, w, b, z, a, Bt, H, W, dil, sgn);
 }
 
@@ -405,8 +420,7 @@ void wgrad(const __nv_bfloat16 *in, const __nv_bfloat16 *g, float *dw, float *db
            cudaStream_t s)
 {
     const int items = Bt * H * ((W + XS - 1) / XS);
-    k_conv_wgrad<C, N><<<std::min(items, 3 * sms()), 288, XS * N * 2 + rows_smem(C, dil), s>>>(in, g, dw, db, Bt, H, W,
-                                                                                              dil);
+    k_conv_wgrad<C, N><<<std::min(items, 3 * sms()), 288, wgrad_smem(C, N, dil), s>>>(in, g, dw, db, Bt, H, W, dil);
 }
 
 void wgrad_any(int C, int N, const __nv_bfloat16 *in, const __nv_bfloat16 *g, float *dw, float *db, int Bt, int H,
