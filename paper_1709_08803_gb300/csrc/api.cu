@@ -164,7 +164,7 @@ int bfs_setup(const bfs_mesh *mesh, const bfs_topo *topo, double F, const bfs_op
     c->plan64 = bfs::plan64_fine(c->Nt, c->Ns, o.src_splits, sms);
     if (o.src_splits <= 0) {
         // FP32C: down to one chunk of sources per split while the split partial
-        // sums stay below 2^20 target slots (40 MB): many short CTAs, so that the
+        // sums stay below 2^20 target slots (25 MB): many short CTAs, so that the
         // last wave of the launch is a small part of it (the split count changes
         // only how the chunk totals are grouped: a two-sum within a split, FP64
         // across splits; the 181 x 61 residuals came out identical)

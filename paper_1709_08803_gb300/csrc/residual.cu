@@ -373,9 +373,9 @@ __device__ __forceinline__ void pair_tile(const double *__restrict__ src, int pe
 // side, one 64-bit word), the target values are broadcast into both halves
 // once per tile, and the offsets are taken target minus source so that no
 // operand needs a negation; the density w g of the bottom double layer is
-// negated while staging for the same reason.  The sums are those of
-// pair_tile<float>: each half accumulates its sources over a chunk, the halves
-// are added and the chunk total enters the two-sum accumulator.
+// negated while staging for the same reason.  Each half accumulates its sources
+// over a chunk in FP32, the halves are added and the chunk total enters the two-sum
+// accumulator of the target.
 // ---------------------------------------------------------------------------
 // Two shared-memory chunk buffers filled by 1-D bulk copies (cp.async.bulk,
 // completion counted in bytes on an mbarrier per buffer): the copy of the
@@ -937,7 +937,7 @@ constexpr int P32_TPB = 128, P32_TPT = 2, P32_CH = 128;
 
 int residual_launch(bfs_ctx *c, const double *u, double *Fu, int precision, cudaStream_t s)
 {
-    // FP32C pairs read the FP32 source records, FP64 and double-float ones the FP64 records
+    // the records of the pair kernel's own arithmetic
     int rc = unpack_launch(c, u, s, precision == BFS_FP32C ? 2 : (precision == BFS_DF64 ? 4 : 1));
     if (rc) return rc;
     const PairPlan &p = precision == BFS_FP32C ? c->plan32 : (precision == BFS_DF64 ? c->plandf : c->plan64);

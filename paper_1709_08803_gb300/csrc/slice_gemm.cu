@@ -151,12 +151,13 @@ __device__ __forceinline__ double sg_scale(double v, int e)
 // C = alpha A B + beta C for a batch of products, 64 x 64 tiles, eight warps of 32 x 16.
 // All S diagonals of a tile stay in registers (16 S a thread), so every slice of a
 // chunk is staged once for its S (S + 1) / 2 products, against shared-memory and
-// L2 traffic of every pair otherwise; that is why the tile is no
-// larger and the sums are mma.sync fragments: in tensor memory nine sums of
-// 128 x 64 would be 576 columns, more than it has.  Copies of the next chunk run
-// (cp.async) under the products of this one.  The 17 products of a 365-row slice take
-// 0.41 ms (1.65 with k_dgemm); one CTA per SM, so the last wave of the 216 to 324
-// tiles is what is left.
+// L2 traffic of every pair otherwise; that is why the tile is no larger.  The sums are
+// mma.sync fragments: in tensor memory nine sums of 128 x 64 would be 576 columns, more
+// than it has; those of 128 x 48 (432 columns) would fit and have not been tried.  Copies
+// of the next chunk run (cp.async) under the products of this one.  The 17 products of a
+// 365-row slice take 0.41 ms (1.65 with k_dgemm).  The tensor pipe is 60 % busy on the SMs
+// that have a tile: 36 for one product (62 us), one CTA each, so that of the 216 to 324
+// tiles of a batch the last wave counts.
 template <int S>
 __global__ void __launch_bounds__(256, 1) k_sg_gemm(SgProds pr, const unsigned short *__restrict__ sl,
                                                     const int *__restrict__ ex, int n, int P, int seg, double alpha,
