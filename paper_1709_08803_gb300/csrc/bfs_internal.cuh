@@ -43,7 +43,7 @@ constexpr int DSRC = 24, DTGT = 20;
 // differences of two of them as they come (pairs_df64.cu); k_records raises d_flag[1]
 // where a node of the residual at hand is higher.  DF_EXACT: vertical distances, in
 // cells, up to which its form for dx == dy is exact; d_flag[2] where one may be larger.
-constexpr double DF_HIGH = 16.0, DF_EXACT = 1447.0;
+constexpr float DF_HIGH = 16.f, DF_EXACT = 1447.f;
 
 // Accumulators written by the pair kernels, per split and target:
 //   0  double and single layers at top targets (top and bottom sheets)

@@ -83,6 +83,7 @@ struct RecArgs {
     int w64, w32, wdf;  // which record copies to write (a residual reads one)
     double x1, y1, dx, dy, sigma, jc, ry;
     double idx, i2dy;  // 1 / dx, 1 / (2 dy)
+    float df_lim;      // so that heights of both sheets and 1 / dx add up to DF_EXACT
 };
 
 // hi + lo float pair of v
@@ -168,9 +169,9 @@ k_records(double *nodal, const double *__restrict__ beta, const double *__restri
             d[44] = (float)c;
             d[46] = 0.f;
             // form: every writer's value is 1
-            const double lim = 0.5 * (DF_EXACT - a.idx);  // so that zeta, beta and 1/dx add up to DF_EXACT
-            if (e < a.Ns && !(fabs(r[2]) <= DF_HIGH && fabs(r[3]) <= DF_HIGH)) form[0] = 1;
-            if (e < a.Ns && !(fabs(r[2]) <= lim && fabs(r[3]) <= lim)) form[1] = 1;
+            const float hz = fabsf((float)r[2]), hb = fabsf((float)r[3]);
+            if (e < a.Ns && !(hz <= DF_HIGH && hb <= DF_HIGH)) form[0] = 1;
+            if (e < a.Ns && !(hz <= a.df_lim && hb <= a.df_lim)) form[1] = 1;
         }
         return;
     }
@@ -213,9 +214,11 @@ k_records(double *nodal, const double *__restrict__ beta, const double *__restri
         o[1] = (float)r[15];
 #pragma unroll
         for (int k = 0; k < 8; k++) split2(v[k], o[2 + 2 * k], o[3 + 2 * k]);
-        // (zeta_x* s + zeta_y* t)^2 no larger than s^2 + t^2, or the sum within DF_EXACT
-        const double my = zys * a.ry, reach = fabs(zxs) * (N - 1) + fabs(my) * (a.half ? 2 * (M - 1) : M - 1);
-        if (!(zxs * zxs + my * my <= 0.99 || reach <= DF_EXACT)) form[1] = 1;
+        // (zeta_x* s + zeta_y* t)^2 no larger than s^2 + t^2, or the sum within DF_EXACT; in
+        // FP32, so that the FP64 operations of the records stay as they are
+        const float mx = fabsf((float)v[6]), my = fabsf((float)v[7]);
+        const float reach = mx * (float)(N - 1) + my * (float)(a.half ? 2 * (M - 1) : M - 1);
+        if (!(mx * mx + my * my <= 0.99f || reach <= DF_EXACT)) form[1] = 1;
     }
 }
 
@@ -856,6 +859,7 @@ static RecArgs rec_args(const bfs_ctx *c)
     a.i2dy = 1.0 / (2.0 * c->dy);
     a.w64 = a.w32 = 1;
     a.wdf = 0;
+    a.df_lim = (float)(0.5 * (DF_EXACT - a.idx));
     return a;
 }
 
