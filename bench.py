@@ -40,8 +40,8 @@ MUFU_PER_INDEX_PAIR = 5  # reciprocal square roots per (target, source) index pa
 # 181x61 from an ncu capture of the current kernel
 PAIRS_TRAFFIC = 1.4336e6  # profiles/k_pairs_181x61.md (43 x 87 CTAs)
 # dram__bytes_read.sum + dram__bytes_write.sum of one FP32 sweep launch at
-# 181x61 from an ncu capture of the current kernel; None until captured
-APPLY_TRAFFIC = None  # not captured since phi_x is eliminated from the blocks
+# 181x61 from an ncu capture of the current kernel
+APPLY_TRAFFIC = 227.7e6  # profiles/k_apply_sweep_181x61.md
 
 
 def _pc_prec(args):
