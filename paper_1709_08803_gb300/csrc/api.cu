@@ -388,7 +388,9 @@ int bfs_precond_apply(bfs_ctx *c, const double *r, double *z, void *stream)
 int bfs_solve(bfs_ctx *c, double *u, bfs_stats *st, void *stream)
 {
     if (!c || !u) return set_err(c, BFS_EINVAL, "NULL argument");
+    if (st) *st = bfs_stats{};
     int rc = bfs::solve_device(c, u, st, (cudaStream_t)stream);
+    if (st) st->status = rc;  // a call that ended before its first residual too
     if (rc && c->err.empty()) {
         const char *m = rc == BFS_ENOCONV ? "Newton iteration limit reached"
                         : rc == BFS_ELINESEARCH ? "line search failed"

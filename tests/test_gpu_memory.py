@@ -52,6 +52,7 @@ for size in (None, 40, 130, 178):  # None loads the kernels
         hog = leave(size * MB)
         for _ in range(2):  # the second call finds nothing half allocated
             no_memory(ctx.solve, u)
+            assert ctx.solve(u, raise_on_error=False)["status"] == bfs.BFS_ENOMEM
         del hog
         torch.cuda.empty_cache()
     assert ctx.solve(u)["status"] == bfs.BFS_OK
